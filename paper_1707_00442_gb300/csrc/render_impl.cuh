@@ -1081,6 +1081,12 @@ shw_status render_f16_big(int mode, int interp, const shw_volume &v, const shw_v
 // the staged marcher (render_slab.cu); SHW_EUNSUPPORTED if it does not apply
 shw_status render_slab(int mode, int interp, const shw_volume &v, const shw_camera &cam, const RenderArgs &a,
                        cudaStream_t st);
+// in-ray smoothing by the rolling marcher (render_roll_taps.cu, render_roll_box.cu); SHW_EUNSUPPORTED
+// if it does not apply
+shw_status render_roll_taps(int mode, int interp, const shw_volume &v, const shw_camera &cam, const RenderArgs &a,
+                            cudaStream_t st);
+shw_status render_roll_box(int mode, int interp, const shw_volume &v, const shw_camera &cam, const RenderArgs &a,
+                           cudaStream_t st);
 // the plane sweep for orthographic spectral-axis views (render_axis.cu); SHW_EUNSUPPORTED if it does not apply
 shw_status render_axis(int mode, int interp, const shw_volume &v, const shw_camera &cam, const RenderArgs &a,
                        cudaStream_t st);

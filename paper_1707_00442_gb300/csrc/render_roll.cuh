@@ -1,0 +1,863 @@
+// render_roll.cuh -- the rolling marcher: in-ray smoothing (Algorithms 8-9) from a ring of
+// cube planes in shared memory.
+//
+// A smoothed sample is up to 25 trilinear fetches around one point.  Gathered from global
+// memory (render_impl.cuh) each fetch is 8 loads whose 32 lanes lie in up to 24-32 different
+// cache lines, and the L1 pipe bounds the kernel.  Here a CTA owns a 16 x 16 pixel tile and
+// its rays advance together along the tile's major axis, a few planes of cells (a step) at a
+// time, while one producer warp keeps the planes that the step's samples and taps can touch
+// in shared memory:
+//   - plane q of the ring holds the cells [oa, oa + wa) x [ob, ob + wb) of that plane, the
+//     tile's footprint there widened by the taps' reach; every plane has its own origin, so
+//     the window follows oblique rays and a plane is staged once per tile;
+//   - a table of plane offsets (pb) turns (plane, a, b) into a shared-memory address;
+//   - one tensor copy brings a plane (a slot of 4 planes for x-major tiles, whose planes are
+//     strided in memory), or one bulk copy per row when the cube's rows are no 16-byte
+//     multiple: row pitch and plane offset then keep every element's global and shared
+//     address equal modulo 16 bytes.
+// Positions, cells, interpolation, the order of the taps and the transfer functions are the
+// gather marcher's, so the results are bit-identical to it.  A sample whose cells are not
+// all staged (a footprint wider than the ring's planes) reads global memory; staging decides
+// the speed, never the result.
+#pragma once
+
+#include "render_slab.cuh"
+
+namespace shw {
+
+enum : int {
+    kRollTaps = 0,  // per-axis taps (Algorithm 9)
+    kRollBox = 1    // the box along the ray on the sample lattice (Algorithm 8, step 1/2)
+};
+
+constexpr int kRollBars = 4;        // headers and barriers: posts in flight
+constexpr int kRollTable = 64;      // entries of the plane table (a power of two)
+constexpr int kRollMaxSlots = 32;   // one producer lane per slot of a window
+constexpr int kRollXG = 4;          // planes per slot of x-major tiles (16-byte rows)
+constexpr int kRollMinBlocks = 2;
+constexpr int kRollBudget2 = 110 * 1024, kRollBudget1 = 222 * 1024;  // bytes of shared memory: two CTAs per SM, one
+
+struct RollHdr {
+    int type, tile;
+    int major, dir;
+    int m0, s_len;            // the step: cells [m0, m0 + s_len) along the major axis
+    int alo, acnt, blo, bcnt; // lateral cells whose samples and taps are all staged
+    int pad[2];
+};
+
+// Staging geometry of one major axis.
+struct RollGeom {
+    int on;      // tiles may take this major axis
+    int g;       // planes per slot
+    int ns;      // slots of the ring
+    int s;       // cells per step, a multiple of g
+    int depth;   // steps staged ahead
+    int wa, wb;  // box extents along the lateral axes A and B
+    int sb;      // floats between rows along B (along A: 1, or g for x-major)
+    int slot;    // floats per slot
+};
+
+struct RollArgs {
+    const float *cube;
+    unsigned *ctr, *err;
+    int ntiles, polls;
+    int halo;       // cells a tap reaches beyond its sample's cell, on each side
+    int rows;       // 1: bulk copies of single rows (ragged or unaligned cube)
+    int goff;       // rows: floats from the 16-byte boundary below the cube to the cube
+    int smem_stage; // bytes of the plane ring
+    int box_mask;   // box: entries of a ray's ring of raw samples, less one (a power of two)
+    RollGeom geo[3];
+};
+
+// One tensor map per major axis (x: slots of 4 x planes; y, z: one plane).
+struct RollMaps {
+    CUtensorMap m[3];
+};
+
+struct RollShared {
+    RollHdr hdr[kRollBars];
+    uint64_t full[kRollBars], empty[kRollBars];
+    int pb[kRollTable];                   // plane q: stage index of its element (a, b) = (0, 0)
+    int oa[kRollTable], ob[kRollTable];   // slot c: origin of its box
+    int quit;
+    int pad[3];
+};
+
+// Lateral axes of major axis M: A (contiguous in the stage) and B.
+template <int M>
+struct RollAxes {
+    static constexpr int A = M == 0 ? 1 : 0;
+    static constexpr int B = M == 2 ? 1 : 2;
+    static constexpr int SA = M == 0 ? kRollXG : 1;  // floats between neighbours along A
+};
+
+// The major axis: the one the tile's rays advance along fastest, so that lateral slopes stay
+// near 1 and the footprint of a plane small.
+__host__ __device__ __forceinline__ TileRays roll_rays(const shw_camera &c, int px0, int py0, const int on[3])
+{
+    TileRays t;
+    for (int i = 0; i < 4; ++i)
+        corner_ray(c, px0 + (i & 1) * (kSlabTW - 1), py0 + (i >> 1) * (kSlabTH - 1), t.o[i], t.u[i]);
+    float best = -1.0f;
+    t.major = 2;
+    t.dir = 1;
+    for (int k = 0; k < 3; ++k) {
+        const float s = t.u[0][k] + t.u[1][k] + t.u[2][k] + t.u[3][k];
+        if (on[k] && fabsf(s) > best) {
+            best = fabsf(s);
+            t.major = k;
+            t.dir = s > 0.0f ? 1 : -1;
+        }
+    }
+    return t;
+}
+
+// Lateral positions [lo, hi] on axis AX of the tile's rays between planes m0 and m1.
+template <int M, int AX>
+__host__ __device__ __forceinline__ void lateral_pos(const TileLines<M> &t, float m0, float m1, float &lo, float &hi)
+{
+    lo = INFINITY;
+    hi = -INFINITY;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const float p0 = t.B[i][AX] * m0 + t.A[i][AX], p1 = t.B[i][AX] * m1 + t.A[i][AX];
+        lo = fminf(lo, fminf(p0, p1));
+        hi = fmaxf(hi, fmaxf(p0, p1));
+    }
+    const float eps = 0.02f + 1e-5f * fmaxf(fabsf(lo), fabsf(hi));
+    lo -= eps;
+    hi += eps;
+}
+
+// Elements [lo, hi] along axis AX that planes [q0, q1] must hold: the corners of the samples
+// next to them widened by the taps' reach H, and the corners of the samples whose taps along
+// the major axis reach them; clipped to the cube.
+template <int M, int AX>
+__host__ __device__ __forceinline__ void plane_extent(const TileLines<M> &t, int q0, int q1, int H, int n, int &lo,
+                                                      int &hi)
+{
+    float l0, h0, l1, h1;
+    lateral_pos<M, AX>(t, (float)(q0 - 1), (float)(q1 + 1), l0, h0);
+    lateral_pos<M, AX>(t, (float)(q0 - 1 - H), (float)(q1 + 1 + H), l1, h1);
+    const float l = fminf(l0 - (float)H, l1), h = fmaxf(h0 + (float)H, h1);
+    lo = (int)floorf(fminf(fmaxf(l, 0.0f), (float)n));
+    hi = (int)floorf(fmaxf(fminf(h + 1.0f, (float)(n - 1)), -1.0f));
+}
+
+// ---- producer -------------------------------------------------------------------------
+
+__device__ __forceinline__ void mbar_expect_tx(uint64_t *bar, uint32_t bytes)
+{
+    asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
+                 : "memory");
+}
+
+// untiled bulk copy: both addresses 16-byte aligned, bytes a multiple of 16
+__device__ __forceinline__ void bulk_load(void *dst, const void *src, uint32_t bytes, uint64_t *bar)
+{
+    asm volatile(
+        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_u32(dst)),
+        "l"(src), "r"(bytes), "r"(smem_u32(bar))
+        : "memory");
+}
+
+struct RollRing {
+    RollShared &sh;
+    const RollArgs &ra;
+    int posts = 0, drained = 0;  // posts made; posts known to be consumed by every warp
+    __device__ __forceinline__ bool drain_to(int p)
+    {
+        for (; drained <= p; ++drained)
+            if (!slab_wait(&sh.empty[drained % kRollBars], (uint32_t)((drained / kRollBars) & 1), &sh.quit, ra.err,
+                           ra.polls))
+                return false;
+        return true;
+    }
+    __device__ __forceinline__ bool post_plain(int type, int tile)
+    {
+        if (!drain_to(posts - kRollBars)) return false;
+        const int st = posts % kRollBars;
+        if ((threadIdx.x & 31) == 0) {
+            RollHdr h{};
+            h.type = type;
+            h.tile = tile;
+            sh.hdr[st] = h;
+            mbar_arrive(&sh.full[st]);
+        }
+        __syncwarp();
+        ++posts;
+        return true;
+    }
+};
+
+__device__ __forceinline__ int floor_div(int a, int b)
+{
+    const int q = a / b;
+    return q * b > a ? q - 1 : q;
+}
+
+// One row's elements [x, x + len) of the cube (len clipped to the row) from row start index
+// `row` into the stage at element index `at` of x: 16-byte pieces by a bulk copy, and at the
+// two ends of the whole cube, where a piece would leave it, single elements.
+__device__ __forceinline__ void roll_row(const RollArgs &ra, float *stage, long long nvox, long long row, int x, int len,
+                                         int at, uint64_t *bar)
+{
+    const long long g0 = ra.goff + row + x, g1 = g0 + len;  // floats from the 16-byte boundary
+    const float *base = ra.cube - ra.goff;
+    long long c0 = g0 & ~3LL, c1 = (g1 + 3) & ~3LL;
+    bool wrote = false;
+    if (c0 < ra.goff) {
+        c0 += 4;
+        for (long long g = g0; g < min(c0, g1); ++g) stage[at + (int)(g - g0)] = __ldg(base + g);
+        wrote = true;
+    }
+    if (c1 > ra.goff + nvox) {
+        c1 -= 4;
+        for (long long g = max(c1, g0); g < g1; ++g) stage[at + (int)(g - g0)] = __ldg(base + g);
+        wrote = true;
+    }
+    if (c1 > c0) {
+        const uint32_t bytes = (uint32_t)(c1 - c0) * 4u;
+        mbar_expect_tx(bar, bytes);
+        bulk_load(stage + at + (int)(c0 - g0), base + c0, bytes, bar);
+    }
+    if (wrote) fence_proxy_async();  // a later bulk copy writes the same bytes
+}
+
+template <int M>
+__device__ __forceinline__ bool roll_produce(const TileRays &r, bool persp, const CUtensorMap *map,
+                                             const RenderArgs &a, const RollArgs &ra, int tile, float *stage,
+                                             RollRing &ring)
+{
+    using AX = RollAxes<M>;
+    TileLines<M> L;
+    if (!tile_lines<M>(r, L)) return true;  // no steps: the consumers read global memory
+    const RollGeom &G = ra.geo[M];
+    RollShared &sh = ring.sh;
+    const int lane = threadIdx.x & 31, dir = r.dir, H = ra.halo;
+    const int n[3] = {a.nx, a.ny, a.nz};
+    const int n_m = n[M], n_a = n[AX::A], n_b = n[AX::B];
+    const int g = M == 0 ? kRollXG : 1, s = G.s;
+    int lo_c = -1, hi_c = n_m - 1;
+    if (persp) {  // every sample lies beyond the eye
+        const int e = (int)fminf(fmaxf(floorf(r.o[0][M]), -1.0f), (float)n_m);
+        if (dir > 0)
+            lo_c = max(lo_c, e);
+        else
+            hi_c = min(hi_c, e);
+    }
+    // the cells [first, last] at which the tile's rays are inside the cube
+    int first = n_m, last = -2;
+    for (int c = lo_c; c <= hi_c; c += 32) {
+        const int cc = c + lane;
+        float al, ah, bl, bh;
+        lateral_pos<M, AX::A>(L, (float)cc, (float)(cc + 1), al, ah);
+        lateral_pos<M, AX::B>(L, (float)cc, (float)(cc + 1), bl, bh);
+        const bool in = cc <= hi_c && ah >= -0.5f && al <= (float)n_a - 0.5f && bh >= -0.5f && bl <= (float)n_b - 0.5f;
+        const unsigned m = __ballot_sync(0xffffffffu, in);
+        if (m) {
+            first = min(first, c + __ffs(m) - 1);
+            last = max(last, c + 31 - __clz(m));
+        }
+    }
+    if (first > last) return true;
+    const int before = ring.posts - 2;  // the last post before this tile's start: it may read the ring
+    bool fresh = true;
+    int have_lo = 0, have_hi = -1;  // slots staged
+    for (int m0 = floor_div(dir > 0 ? first : last, s) * s; dir > 0 ? m0 <= last : m0 + s > first; m0 += dir * s) {
+        const int plo = max(m0 - H, 0), phi = min(m0 + s + H, n_m - 1);
+        const int slo = plo / g, shi = phi / g;
+        const int c0 = fresh ? slo : (dir > 0 ? have_hi + 1 : slo), c1 = fresh ? shi : (dir > 0 ? shi : have_lo - 1);
+        // the slots overwritten now were last read `depth` steps ago (or by the tile before)
+        if (!ring.drain_to(max(ring.posts - kRollBars, fresh ? before : ring.posts - 1 - G.depth))) return false;
+        const int st = ring.posts % kRollBars;
+        uint64_t *bar = &sh.full[st];
+        const int cnt = max(c1 - c0 + 1, 0);
+        int oa = 0, ob = 0;
+        if (lane < cnt) {
+            const int c = c0 + lane, q0 = c * g;
+            int lo, hi;
+            plane_extent<M, AX::A>(L, q0, q0 + g - 1, H, n_a, lo, hi);
+            if (hi - lo + 1 > G.wa) lo += (hi - lo + 1 - G.wa) >> 1;
+            oa = min(max(lo, 0), n_a - 1);
+            if (M != 0 && !ra.rows) oa &= ~3;  // a tensor copy's x start: 16 bytes
+            plane_extent<M, AX::B>(L, q0, q0 + g - 1, H, n_b, lo, hi);
+            if (hi - lo + 1 > G.wb) lo += (hi - lo + 1 - G.wb) >> 1;
+            ob = min(max(lo, 0), n_b - 1);
+            sh.oa[c & (kRollTable - 1)] = oa;
+            sh.ob[c & (kRollTable - 1)] = ob;
+            int pb = (c % G.ns) * G.slot - oa * AX::SA - ob * G.sb;
+            if (M != 0 && ra.rows) {
+                // equal global and shared addresses modulo 16 bytes (the row pitch agrees already)
+                const int want = ra.goff + (M == 2 ? (c * n[1] & 3) * (n[0] & 3) : (c & 3) * (n[0] & 3));
+                pb += 4 + ((want - pb) & 3);
+            }
+#pragma unroll
+            for (int j = 0; j < g; ++j) sh.pb[(q0 + j) & (kRollTable - 1)] = pb + j;
+        }
+        __syncwarp();
+        if (M == 0 || !ra.rows) {
+            if (lane < cnt) {
+                const int c = c0 + lane;
+                float *dst = stage + (size_t)(c % G.ns) * G.slot;
+                if (tma_dst_ok(dst, ra.err)) {  // always: slots are 128-byte multiples
+                    mbar_expect_tx(bar, (uint32_t)(G.wa * G.wb * g * 4));
+                    if constexpr (M == 0)
+                        tma_load_3d(dst, map, c * g, oa, ob, bar);
+                    else if constexpr (M == 1)
+                        tma_load_3d(dst, map, oa, c, ob, bar);
+                    else
+                        tma_load_3d(dst, map, oa, ob, c, bar);
+                }
+            }
+        } else {
+            const long long nvox = (long long)n[0] * n[1] * n[2];
+            for (int i = lane; i < cnt * G.wb; i += 32) {
+                const int c = c0 + i / G.wb, ci = c & (kRollTable - 1);
+                const int b = sh.ob[ci] + i % G.wb, x = sh.oa[ci];
+                if (b >= n_b) continue;
+                const long long row = M == 2 ? ((long long)c * n[1] + b) * n[0] : ((long long)b * n[1] + c) * n[0];
+                roll_row(ra, stage, nvox, row, x, min(G.wa, n_a - x), sh.pb[ci] + b * G.sb + x, bar);
+            }
+        }
+        // the lateral cells whose samples and taps every plane of the window holds
+        int alo = -1, ahi = n_a - 1, blo = -1, bhi = n_b - 1;
+        if (slo + lane <= shi) {
+            const int c = slo + lane, ci = c & (kRollTable - 1), q0 = c * g;
+            const bool own = q0 + g - 1 >= m0 && q0 <= m0 + s;  // planes of the step's own cells
+            const int h = own ? H : 0, x = sh.oa[ci], y = sh.ob[ci];
+            if (x > 0) alo = x + h;
+            if (x + G.wa < n_a) ahi = x + G.wa - 2 - h;
+            if (y > 0) blo = y + h;
+            if (y + G.wb < n_b) bhi = y + G.wb - 2 - h;
+        }
+        alo = __reduce_max_sync(0xffffffffu, alo);
+        ahi = __reduce_min_sync(0xffffffffu, ahi);
+        blo = __reduce_max_sync(0xffffffffu, blo);
+        bhi = __reduce_min_sync(0xffffffffu, bhi);
+        if (lane == 0) {
+            RollHdr h;
+            h.type = kStageSlab;
+            h.tile = tile;
+            h.major = M;
+            h.dir = dir;
+            h.m0 = m0;
+            h.s_len = s;
+            h.alo = alo;
+            h.acnt = max(ahi - alo + 1, 0);
+            h.blo = blo;
+            h.bcnt = max(bhi - blo + 1, 0);
+            sh.hdr[st] = h;
+        }
+        __syncwarp();  // every lane's expected bytes and table entries come before the arrival
+        if (lane == 0) mbar_arrive(bar);
+        ++ring.posts;
+        fresh = false;
+        have_lo = slo;
+        have_hi = shi;
+    }
+    return true;
+}
+
+__device__ __forceinline__ void roll_producer(const CUtensorMap *maps, const shw_camera &cam, const RenderArgs &a,
+                                              const RollArgs &ra, float *stage, RollShared &sh)
+{
+    const int lane = threadIdx.x & 31;
+    RollRing ring{sh, ra};
+    const int on[3] = {ra.geo[0].on, ra.geo[1].on, ra.geo[2].on};
+    bool ok = true;
+    while (ok) {
+        unsigned t = 0;
+        if (lane == 0) t = atomicAdd(ra.ctr, 1u);
+        t = __shfl_sync(0xffffffffu, t, 0);
+        if (t >= (unsigned)ra.ntiles) {
+            ring.post_plain(kStageExit, 0);
+            break;
+        }
+        if (!ring.post_plain(kStageTile, (int)t)) break;
+        int tx, ty;
+        slab_tile((int)t, a, tx, ty);
+        const TileRays r = roll_rays(cam, tx * kSlabTW, ty * kSlabTH, on);
+        const bool persp = !cam.ortho;
+        if (r.major == 0)
+            ok = roll_produce<0>(r, persp, &maps[0], a, ra, (int)t, stage, ring);
+        else if (r.major == 1)
+            ok = roll_produce<1>(r, persp, &maps[1], a, ra, (int)t, stage, ring);
+        else
+            ok = roll_produce<2>(r, persp, &maps[2], a, ra, (int)t, stage, ring);
+        if (ok) ok = ring.post_plain(kStageTileEnd, (int)t);
+    }
+    // no exit while a copy into this CTA's shared memory is in flight: wait (bounded) for the
+    // last posts
+    if (lane == 0) {
+        for (int i = max(0, ring.posts - kRollBars); i < ring.posts; ++i)
+            for (int it = 0; it < ra.polls && !mbar_try_wait_sleep(&sh.full[i % kRollBars],
+                                                                   (uint32_t)((i / kRollBars) & 1), kSlabSleepNs);
+                 ++it) {
+            }
+    }
+    __syncwarp();
+}
+
+// ---- consumer -------------------------------------------------------------------------
+
+// One axis of a fetch: the two corner indexes and the weight.  CLAMP: indexes clamp to the
+// edge voxel (the gather marcher's rule); without it the cell lies inside the cube.
+template <bool CLAMP>
+__device__ __forceinline__ void roll_axis(long long p, int n, int &i0, int &i1, float &f)
+{
+    const int c = cell_of<CLAMP>(p, n);
+    i0 = CLAMP ? max(c, 0) : c;
+    i1 = CLAMP ? min(c + 1, n - 1) : c + 1;
+    f = fx_frac(p);
+}
+
+// The value at (PA, PB, PM): the trilinear sample, and with TAPS its chain of taps along x,
+// then y, then z (smoothed_sample's order and arithmetic), from the staged planes.
+template <int M, bool CLAMP, bool TAPS>
+__device__ __forceinline__ float roll_value(const float *stage, const int *pbt, int sb, int lim, const int n[3],
+                                            const long long P[3], const RenderArgs &a)
+{
+    using AX = RollAxes<M>;
+    constexpr int A = AX::A, B = AX::B, SA = AX::SA;
+    int i0[3], i1[3];
+    float f[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) roll_axis<CLAMP>(P[k], n[k], i0[k], i1[k], f[k]);
+    auto plane = [&](int q) { return pbt[q & (kRollTable - 1)]; };
+    // corners c[x + 2 y + 4 z] from plane offsets m0, m1 and in-plane offsets
+    auto fetch8 = [&](int m0, int m1, int a0, int a1, int b0, int b1, float fx, float fy, float fz) {
+        if constexpr (kChecked) {  // every corner lies in the stage (lim floats)
+            const int l0 = min(min(m0, m1) + b0, min(m0, m1) + b1) + a0, l1 = max(m0, m1) + max(b0, b1) + a1;
+            const bool ok = l0 >= 0 && l1 < lim;
+            SHW_CHECK(ok);
+            if (!ok) m0 = m1 = a0 = a1 = b0 = b1 = 0;
+        }
+        const float *p00 = stage + (m0 + b0), *p01 = stage + (m0 + b1), *p10 = stage + (m1 + b0),
+                    *p11 = stage + (m1 + b1);
+        float c[8];
+#define SHW_C(m, b, x, ptr, off) c[((m) << M) | ((b) << B) | ((x) << A)] = (ptr)[off]
+        SHW_C(0, 0, 0, p00, a0);
+        SHW_C(0, 0, 1, p00, a1);
+        SHW_C(0, 1, 0, p01, a0);
+        SHW_C(0, 1, 1, p01, a1);
+        SHW_C(1, 0, 0, p10, a0);
+        SHW_C(1, 0, 1, p10, a1);
+        SHW_C(1, 1, 0, p11, a0);
+        SHW_C(1, 1, 1, p11, a1);
+#undef SHW_C
+        return trilerp(c, fx, fy, fz);
+    };
+    const int m0 = plane(i0[M]), m1 = plane(i1[M]);
+    const int a0 = i0[A] * SA, a1 = CLAMP ? i1[A] * SA : a0 + SA;
+    const int b0 = i0[B] * sb, b1 = CLAMP ? i1[B] * sb : b0 + sb;
+    float v = fetch8(m0, m1, a0, a1, b0, b1, f[0], f[1], f[2]);
+    if constexpr (TAPS) {
+#pragma unroll
+        for (int ax = 0; ax < 3; ++ax) {
+            float out = v * a.smooth_c0;
+            for (int j = 0; j < a.smooth_n; ++j) {
+                const long long off = a.smooth_off[j];
+                const float w = a.smooth_w[j];
+#pragma unroll
+                for (int sgn = 0; sgn < 2; ++sgn) {
+                    int t0, t1;
+                    float tf;
+                    roll_axis<CLAMP>(sgn == 0 ? P[ax] + off : P[ax] - off, n[ax], t0, t1, tf);
+                    float t;
+                    if (ax == M) {
+                        t = fetch8(plane(t0), plane(t1), a0, a1, b0, b1, M == 0 ? tf : f[0], M == 1 ? tf : f[1],
+                                   M == 2 ? tf : f[2]);
+                    } else if (ax == A) {
+                        const int u0 = t0 * SA, u1 = CLAMP ? t1 * SA : u0 + SA;
+                        t = fetch8(m0, m1, u0, u1, b0, b1, A == 0 ? tf : f[0], A == 1 ? tf : f[1], f[2]);
+                    } else {
+                        const int u0 = t0 * sb, u1 = CLAMP ? t1 * sb : u0 + sb;
+                        t = fetch8(m0, m1, a0, a1, u0, u1, f[0], B == 1 ? tf : f[1], B == 2 ? tf : f[2]);
+                    }
+                    out = __fmaf_rn(t, w, out);
+                }
+            }
+            v = out;
+        }
+    }
+    return v;
+}
+
+// The same value from global memory (a sample that the ring does not hold).  Not inlined:
+// rare, and its registers would add to the staged path's.
+template <bool TAPS, class S>
+__device__ __noinline__ float roll_global(const S &s, long long X, long long Y, long long Z, const RenderArgs &a)
+{
+    CellCache cc;
+    if constexpr (TAPS) {
+        const long long U[3] = {0, 0, 0};
+        return smoothed_sample<SHW_TRILINEAR>(s, X, Y, Z, U, a, cc);
+    } else {
+        return s.trilinear(X, Y, Z);
+    }
+}
+
+// One ray's march: its raw samples arrive in order, k = 0 .. N-1 (taps) or, for the box,
+// k = -2 arm .. N-1 + 2 arm.
+template <int MODE, int KIND>
+struct RollMarch {
+    using St = typename StateOf<MODE>::type;
+    St st;
+    long long X, Y, Z;  // position of sample k
+    int k, kend;        // next sample, end of the samples
+    int ka, kb;         // samples whose cells and taps need no clamping
+    int done;           // samples processed
+    float s0, s1;       // box: running sums of the classes of the next sample and the one after
+
+    // Take value v of sample k; true if the transfer function stopped the ray.
+    __device__ __forceinline__ bool take(const RenderArgs &a, float v, float *ring, int mask)
+    {
+        if constexpr (KIND == kRollTaps) {
+            v = filter_value(isnan(v) ? a.lo : v, a);
+            v = isnan(v) ? a.lo : v;  // a NaN sample counts as DATAMIN
+            done = k + 1;
+            return st.update(v, k);
+        } else {
+            // march_box_lattice's recurrence (M = 2), its raw samples kept in the ray's ring
+            const int arm = a.smooth_n, j = k, c = j - 2 * arm;
+            auto at = [&](int i) -> float & { return ring[(i & mask) * (32 * kSlabWarps)]; };
+            at(j) = v;
+            if (c < 0) return false;
+            float t = 0.0f;
+            bool direct = (c >> 1) % SHW_BOX_RESUM == 0;
+            if (!direct) {
+                t = s0 + v - at(j - (4 * arm + 2));
+                direct = !isfinite(t);
+            }
+            if (direct) {  // the definition's order: the sample, then the pairs +-i
+                t = at(c);
+                for (int i = 1; i <= arm; ++i) {
+                    t += at(c + 2 * i);
+                    t += at(c - 2 * i);
+                }
+            }
+            s0 = s1;
+            s1 = t;
+            float w = t * a.smooth_c0;
+            w = filter_value(isnan(w) ? a.lo : w, a);
+            w = isnan(w) ? a.lo : w;
+            done = c + 1;
+            return st.update(w, c);
+        }
+    }
+};
+
+// The samples of one ray in the step of h; true if the transfer function stopped the ray.
+template <int M, int MODE, int KIND, class S>
+__device__ __forceinline__ bool roll_step(const S &s, const RenderArgs &a, RollMarch<MODE, KIND> &q, long long DX,
+                                          long long DY, long long DZ, const RollHdr &h, const float *stage,
+                                          const int *pbt, int sb, int lim, float *ring, int mask)
+{
+    using AX = RollAxes<M>;
+    const int n[3] = {s.nx, s.ny, s.nz};
+    const int m_edge = h.dir > 0 ? h.m0 : h.m0 + h.s_len - 1;
+    while (q.k < q.kend) {
+        const long long P[3] = {q.X, q.Y, q.Z};
+        const int cm = clampi(fx_cell(P[M]), -1, n[M] - 1);
+        const int rel = h.dir > 0 ? cm - m_edge : m_edge - cm;
+        if (rel >= h.s_len) return false;  // a later step's
+        const int ca = clampi(fx_cell(P[AX::A]), -1, n[AX::A] - 1), cb = clampi(fx_cell(P[AX::B]), -1, n[AX::B] - 1);
+        float v;
+        if (rel >= 0 && (unsigned)(ca - h.alo) < (unsigned)h.acnt && (unsigned)(cb - h.blo) < (unsigned)h.bcnt) {
+            if (q.k >= q.ka && q.k < q.kb)
+                v = roll_value<M, false, KIND == kRollTaps>(stage, pbt, sb, lim, n, P, a);
+            else
+                v = roll_value<M, true, KIND == kRollTaps>(stage, pbt, sb, lim, n, P, a);
+        } else {
+            v = roll_global<KIND == kRollTaps>(s, q.X, q.Y, q.Z, a);
+        }
+        const bool stop = q.take(a, v, ring, mask);
+        q.X += DX;
+        q.Y += DY;
+        q.Z += DZ;
+        ++q.k;
+        if (stop) return true;
+    }
+    return false;
+}
+
+template <int MODE, int KIND, class S>
+__device__ __forceinline__ void roll_consumer(const S &s, const shw_camera &cam, const RenderArgs &a,
+                                              const RollArgs &ra, const float *stage, RollShared &sh, float *rings)
+{
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int lx = (warp & 1) * 8 + (lane & 7), ly = (warp >> 1) * 4 + (lane >> 3);
+    volatile int *quit = &sh.quit;
+    float *ring = rings + threadIdx.x;
+    RollMarch<MODE, KIND> q;
+    RayFx r;
+    long long pix = 0;
+    int N = 0;
+    bool has = false, live = false;
+    for (int posts = 0;; ++posts) {
+        const int si = posts % kRollBars;
+        if (!slab_wait(&sh.full[si], (uint32_t)((posts / kRollBars) & 1), quit, ra.err, ra.polls)) return;
+        const RollHdr h = sh.hdr[si];
+        if (h.type == kStageExit) return;
+        if (h.type == kStageTile) {
+            int tx, ty;
+            slab_tile(h.tile, a, tx, ty);
+            const int px = tx * kSlabTW + lx, py = ty * kSlabTH + ly;
+            has = px < a.width && py < a.height;
+            pix = (long long)py * a.width + px;
+            const bool hit = has && !quick_miss(cam, px, py, s.nx, s.ny, s.nz) &&
+                             setup_ray(cam, px, py, s.nx, s.ny, s.nz, a.step, r);
+            N = hit ? min(r.N, a.nmax) : 0;
+            live = N > 0;
+            q.st = typename RollMarch<MODE, KIND>::St{};
+            q.done = 0;
+            if (live) {
+                // samples whose cells lie in [H, n - 2 - H] on every axis
+                const int H = ra.halo;
+                RayFx in = r;
+                for (int k = 0; k < 3; ++k) in.P[k] -= (long long)H << 32;
+                interior_range(in, s.nx - 2 * H, s.ny - 2 * H, s.nz - 2 * H, N, q.ka, q.kb);
+                init_ray_state<MODE, SHW_TRILINEAR>(q.st, s, a, r, pix, a.lut);
+                const int lead = KIND == kRollBox ? 2 * a.smooth_n : 0;  // raw samples before the first
+                q.k = -lead;
+                q.kend = N + lead;
+                q.X = r.P[0] - (long long)lead * r.D[0];
+                q.Y = r.P[1] - (long long)lead * r.D[1];
+                q.Z = r.P[2] - (long long)lead * r.D[2];
+                q.s0 = q.s1 = 0.0f;
+            }
+        } else if (h.type == kStageSlab) {
+            if (live) {
+                bool stop;
+                if (h.major == 0)
+                    stop = roll_step<0, MODE, KIND>(s, a, q, r.D[0], r.D[1], r.D[2], h, stage, sh.pb, ra.geo[0].sb,
+                                                    ra.smem_stage / 4, ring, ra.box_mask);
+                else if (h.major == 1)
+                    stop = roll_step<1, MODE, KIND>(s, a, q, r.D[0], r.D[1], r.D[2], h, stage, sh.pb, ra.geo[1].sb,
+                                                    ra.smem_stage / 4, ring, ra.box_mask);
+                else
+                    stop = roll_step<2, MODE, KIND>(s, a, q, r.D[0], r.D[1], r.D[2], h, stage, sh.pb, ra.geo[2].sb,
+                                                    ra.smem_stage / 4, ring, ra.box_mask);
+                if (stop) live = false;
+            }
+        } else if (has) {  // the tile's end
+            if (live) {    // samples that no step held
+                while (q.k < q.kend) {
+                    const float v = roll_global<KIND == kRollTaps>(s, q.X, q.Y, q.Z, a);
+                    const bool stop = q.take(a, v, ring, ra.box_mask);
+                    q.X += r.D[0];
+                    q.Y += r.D[1];
+                    q.Z += r.D[2];
+                    ++q.k;
+                    if (stop) break;
+                }
+                live = false;
+            }
+            if (N <= 0) r.P[0] = r.P[1] = r.P[2] = r.D[0] = r.D[1] = r.D[2] = 0;
+            emit_ray<MODE, SHW_TRILINEAR>(a, pix, N, r.P, r.D, q.st, q.done);
+            has = false;
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&sh.empty[si]);
+    }
+}
+
+template <int MODE, int KIND, class S>
+__global__ void __launch_bounds__(kSlabThreads, kRollMinBlocks)
+    roll_kernel(const __grid_constant__ RollMaps maps, const __grid_constant__ S s,
+                const __grid_constant__ shw_camera cam, const __grid_constant__ RenderArgs a,
+                const __grid_constant__ RollArgs ra)
+{
+    extern __shared__ __align__(128) unsigned char roll_smem[];
+    float *stage = reinterpret_cast<float *>(roll_smem);
+    RollShared &sh = *reinterpret_cast<RollShared *>(roll_smem + ra.smem_stage);
+    float *rings = reinterpret_cast<float *>(roll_smem + ra.smem_stage + sizeof(RollShared));
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < kRollBars; ++i) {
+            mbar_init(&sh.full[i], 1);
+            mbar_init(&sh.empty[i], kSlabWarps);
+        }
+        sh.quit = 0;
+        fence_barrier_init();
+    }
+    __syncthreads();
+    if ((threadIdx.x >> 5) == kSlabWarps)
+        roll_producer(maps.m, cam, a, ra, stage, sh);
+    else
+        roll_consumer<MODE, KIND>(s, cam, a, ra, stage, sh, rings);
+}
+
+// ---- host -----------------------------------------------------------------------------
+
+// Largest plane extents of major axis M over sampled tiles and planes.
+template <int M>
+inline void roll_extent(const TileRays &r, const int n[3], int H, int g, int &wa, int &wb)
+{
+    using AX = RollAxes<M>;
+    TileLines<M> L;
+    if (!tile_lines<M>(r, L)) return;
+    for (int i = 0; i <= 4; ++i) {
+        const int q = (int)((long long)(n[M] - 1) * i / 4) / g * g;
+        int al, ah, bl, bh;
+        plane_extent<M, AX::A>(L, q, q + g - 1, H, n[AX::A], al, ah);
+        plane_extent<M, AX::B>(L, q, q + g - 1, H, n[AX::B], bl, bh);
+        if (al > ah || bl > bh) continue;  // the tile passes the cube here
+        wa = std::max(wa, ah - al + 1);
+        wb = std::max(wb, bh - bl + 1);
+    }
+}
+
+// Slots a step's window spans, with `depth` steps staged ahead.
+inline int roll_slots(int H, int s, int g, int depth) { return (H + g - 1) / g + (s + H) / g + 1 + depth * s / g; }
+
+// The launch's staging geometry: for each major axis that its tiles take, box extents that
+// hold the sampled tiles' footprints, the longest step whose window fits the shared memory
+// budget.  False when no step fits: the gather marcher then serves the request.
+inline bool roll_geometry(const shw_camera &cam, const int n[3], int H, bool tmaps, int budget, int smax, int min_s,
+                          RollArgs &ra)
+{
+    const int on[3] = {tmaps, 1, 1};
+    int wa[3] = {0, 0, 0}, wb[3] = {0, 0, 0};
+    bool used[3] = {false, false, false};
+    const int tx = ceil_div(cam.width, kSlabTW), ty = ceil_div(cam.height, kSlabTH);
+    for (int j = 0; j < 5; ++j)
+        for (int i = 0; i < 5; ++i) {
+            const TileRays r = roll_rays(cam, (int)((long long)(tx - 1) * i / 4) * kSlabTW,
+                                         (int)((long long)(ty - 1) * j / 4) * kSlabTH, on);
+            used[r.major] = true;
+            if (r.major == 0) roll_extent<0>(r, n, H, kRollXG, wa[0], wb[0]);
+            else if (r.major == 1) roll_extent<1>(r, n, H, 1, wa[1], wb[1]);
+            else roll_extent<2>(r, n, H, 1, wa[2], wb[2]);
+        }
+    int stage = 0;
+    bool any = false;
+    for (int M = 0; M < 3; ++M) {
+        RollGeom &G = ra.geo[M];
+        G = RollGeom{};
+        if (!used[M] || wa[M] <= 0 || wb[M] <= 0) {
+            // no sampled tile: a tile that takes this axis all the same reads global memory
+            continue;
+        }
+        const int A = M == 0 ? 1 : 0, B = M == 2 ? 1 : 2;
+        G.g = M == 0 ? kRollXG : 1;
+        G.wb = std::min(wb[M] + 1, n[B]);
+        G.wa = std::min(wa[M] + 1, n[A]);
+        if (M == 0) {
+            G.wa |= 1;  // an odd number of 16-byte rows: neighbours along B on other banks
+            G.sb = G.g * G.wa;
+            G.slot = G.sb * G.wb;
+        } else if (tmaps) {
+            G.wa = (G.wa + 3 + 3) / 4 * 4;      // the box starts on 16 bytes
+            if (G.wa % 8 == 0) G.wa += 4;       // an odd number of 16 bytes per row
+            G.sb = G.wa;
+            G.slot = G.sb * G.wb;
+        } else {
+            const int want = (M == 2 ? n[0] : (n[0] & 3) * (n[1] & 3)) & 3;  // row pitch of the cube modulo 4
+            G.sb = G.wa + 6;
+            G.sb += (want - G.sb) & 3;
+            G.slot = G.sb * G.wb + 16;
+        }
+        if (G.wa > 256 || G.wb > 256) return false;
+        G.slot = (G.slot + 31) & ~31;
+        G.depth = 1;
+        const int cap = std::min(std::min(kRollMaxSlots, kRollTable / G.g), budget / (G.slot * 4));
+        G.s = 0;
+        for (int s = G.g; s <= std::max(smax, G.g); s += G.g)
+            if (roll_slots(H, s, G.g, G.depth) <= cap) G.s = s;
+        if (G.s < std::max(min_s, G.g)) return false;
+        G.ns = roll_slots(H, G.s, G.g, G.depth);
+        G.on = 1;
+        any = true;
+        stage = std::max(stage, G.ns * G.slot * 4);
+    }
+    ra.smem_stage = (stage + 127) & ~127;
+    return any;
+}
+
+template <int MODE, int KIND, class S>
+shw_status roll_launch_one(const RollMaps &maps, const S &s, const shw_camera &cam, const RenderArgs &a,
+                           const RollArgs &ra, size_t smem, cudaStream_t st)
+{
+    auto kern = roll_kernel<MODE, KIND, S>;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+        cudaGetLastError();
+        return SHW_ECUDA;
+    }
+    const int nsm = sm_count(), per_sm = smem <= (size_t)113 * 1024 ? 2 : 1;
+    if (nsm <= 0) return SHW_ECUDA;
+    const long long grid = std::min<long long>((long long)per_sm * nsm, ra.ntiles);
+    kern<<<(unsigned)std::max<long long>(grid, 1), kSlabThreads, smem, st>>>(maps, s, cam, a, ra);
+    return after_launch();
+}
+
+// In-ray smoothing of a float32 cube through the rolling marcher; SHW_EUNSUPPORTED when it
+// does not serve the request.
+template <int KIND>
+shw_status roll_launch(int mode, const shw_volume &v, const shw_camera &cam, const RenderArgs &a0, cudaStream_t st)
+{
+    const SamplerF32<int> s{static_cast<const float *>(v.data), v.nx, v.ny, v.nz, v.nx, v.nx * v.ny};
+    using S = SamplerF32<int>;
+    const int n[3] = {v.nx, v.ny, v.nz};
+    RollArgs ra{};
+    ra.cube = s.v;
+    ra.halo = 0;
+    if (KIND == kRollTaps)  // a tap at offset o reaches cells up to ceil(|o|) away
+        for (int j = 0; j < a0.smooth_n; ++j) {
+            const long long o = a0.smooth_off[j] < 0 ? -a0.smooth_off[j] : a0.smooth_off[j];
+            ra.halo = std::max(ra.halo, (int)((o + 0xffffffffLL) >> 32));
+        }
+    const bool tmaps = v.nx % 4 == 0 && aligned(v.data, 16);
+    ra.rows = !tmaps;
+    ra.goff = (int)((reinterpret_cast<uintptr_t>(v.data) >> 2) & 3);
+    size_t extra = sizeof(RollShared);
+    if (KIND == kRollBox) {
+        int len = 1;
+        while (len < 4 * a0.smooth_n + 3) len *= 2;
+        ra.box_mask = len - 1;
+        extra += (size_t)len * 32 * kSlabWarps * 4;
+    }
+    // two CTAs per SM where a step of at least two cells fits, else one
+    const int smax = KIND == kRollTaps ? 4 : 12;
+    if (!roll_geometry(cam, n, ra.halo, tmaps, kRollBudget2 - (int)extra, smax, 2, ra) &&
+        !roll_geometry(cam, n, ra.halo, tmaps, kRollBudget1 - (int)extra, smax, 1, ra))
+        return SHW_EUNSUPPORTED;
+    RollMaps maps{};
+    if (tmaps) {
+        const RollGeom *G = ra.geo;
+        if ((G[0].on && !encode_tmap_3d(&maps.m[0], s.v, 4, v.nx, v.ny, v.nz, kRollXG, G[0].wa, G[0].wb)) ||
+            (G[1].on && !encode_tmap_3d(&maps.m[1], s.v, 4, v.nx, v.ny, v.nz, G[1].wa, 1, G[1].wb)) ||
+            (G[2].on && !encode_tmap_3d(&maps.m[2], s.v, 4, v.nx, v.ny, v.nz, G[2].wa, G[2].wb, 1)))
+            return SHW_EUNSUPPORTED;
+    }
+    RenderArgs a = a0;
+    a.tiles_x = ceil_div(cam.width, kSlabTW);
+    a.tiles_y = ceil_div(cam.height, kSlabTH);
+    float cpx, cpy;
+    project_centre(cam, v.nx, v.ny, v.nz, cpx, cpy);
+    a.ctx = (int)fminf(fmaxf(cpx / kSlabTW, 0.0f), (float)(a.tiles_x - 1));
+    a.cty = (int)fminf(fmaxf(cpy / kSlabTH, 0.0f), (float)(a.tiles_y - 1));
+    ra.ntiles = a.tiles_x * a.tiles_y;
+    ra.err = device_error_word();
+    ra.polls = kSlabWaitPolls;
+    ra.ctr = work_counter(st);
+    if (!ra.ctr) return SHW_ECUDA;
+    const size_t smem = (size_t)ra.smem_stage + extra;
+    switch (mode) {
+    case SHW_MIP:
+        // without a channel output only the maximum's value matters
+        if (a.index == nullptr) return roll_launch_one<kMipValue, KIND, S>(maps, s, cam, a, ra, smem, st);
+        return roll_launch_one<SHW_MIP, KIND, S>(maps, s, cam, a, ra, smem, st);
+    case SHW_AVG: return roll_launch_one<SHW_AVG, KIND, S>(maps, s, cam, a, ra, smem, st);
+    case SHW_COMPOSITE: return roll_launch_one<SHW_COMPOSITE, KIND, S>(maps, s, cam, a, ra, smem, st);
+    case SHW_SPECTRAL: return roll_launch_one<SHW_SPECTRAL, KIND, S>(maps, s, cam, a, ra, smem, st);
+    case SHW_MOMENT1: return roll_launch_one<SHW_MOMENT1, KIND, S>(maps, s, cam, a, ra, smem, st);
+    case SHW_COMPOSITE_SPECTRAL:
+        return roll_launch_one<SHW_COMPOSITE_SPECTRAL, KIND, S>(maps, s, cam, a, ra, smem, st);
+    case SHW_MIP_RGB: return roll_launch_one<SHW_MIP_RGB, KIND, S>(maps, s, cam, a, ra, smem, st);
+    case SHW_COMPOSITE_RGB: return roll_launch_one<SHW_COMPOSITE_RGB, KIND, S>(maps, s, cam, a, ra, smem, st);
+    default: return SHW_EUNSUPPORTED;
+    }
+}
+
+}  // namespace shw

@@ -109,7 +109,7 @@ struct SlabGeom {
 
 // The ray of pixel centre (px + 1/2, py + 1/2) as origin o and (unnormalised) direction u
 // (Appendix A); pixels beyond the image are allowed (the tile's outer corners).
-__device__ __forceinline__ void corner_ray(const shw_camera &c, int px, int py, float o[3], float u[3])
+__host__ __device__ __forceinline__ void corner_ray(const shw_camera &c, int px, int py, float o[3], float u[3])
 {
     const float W = (float)c.width, H = (float)c.height;
     const float xs = (float)(2 * px + 1 - c.width) / W, ys = (float)(c.height - 2 * py - 1) / H;
@@ -166,7 +166,7 @@ struct TileLines {
 };
 
 template <int M>
-__device__ __forceinline__ bool tile_lines(const TileRays &r, TileLines<M> &t)
+__host__ __device__ __forceinline__ bool tile_lines(const TileRays &r, TileLines<M> &t)
 {
     bool ok = true;
 #pragma unroll
