@@ -11,14 +11,24 @@
 //     tile's footprint there widened by the taps' reach; every plane has its own origin, so
 //     the window follows oblique rays and a plane is staged once per tile;
 //   - a table of plane offsets (pb) turns (plane, a, b) into a shared-memory address;
-//   - one tensor copy brings a plane (a slot of 4 planes for x-major tiles, whose planes are
-//     strided in memory), or one bulk copy per row when the cube's rows are no 16-byte
-//     multiple: row pitch and plane offset then keep every element's global and shared
-//     address equal modulo 16 bytes.
+//   - one tensor copy brings a plane, or one bulk copy per row when the cube's rows are no
+//     16-byte multiple: row pitch and plane offset then keep every element's global and
+//     shared address equal modulo 16 bytes.  The planes of x-major tiles are strided in
+//     memory: the producer warp loads four of them together (16 bytes a row) and transposes
+//     them into planes, which costs 4 % of the samples' own shared-memory traffic;
+//   - the row pitch follows the view: the 32 rays of a warp cross a plane at about 8 x 4
+//     points, and a pitch that puts consecutive rows on consecutive banks keeps them apart.
 // Positions, cells, interpolation, the order of the taps and the transfer functions are the
 // gather marcher's, so the results are bit-identical to it.  A sample whose cells are not
 // all staged (a footprint wider than the ring's planes) reads global memory; staging decides
 // the speed, never the result.
+//
+// What bounds it (512^3 cube, 1000 x 1000 MIP): with 9 taps per axis the shared-memory pipe (92 %
+// of its wavefronts; 104 corner loads a sample at 2.1 wavefronts each, the conflicts of 32
+// rays whose cells fall irregularly on 32 banks; 53.9 ms gathered from global memory, 11.5 ms
+// here); with the box issue slots and latency (50 % of issue; 5.86 -> 2.32 ms).  On the way: one
+// lateral range per step instead of one per cell (4 % of the samples in global memory) 16.8 ms;
+// x-major planes as [z][y][4 x] boxes, unspread over the banks (3.9 wavefronts a load) 18.6 ms.
 #pragma once
 
 #include "render_slab.cuh"
@@ -33,15 +43,14 @@ enum : int {
 constexpr int kRollBars = 4;        // headers and barriers: posts in flight
 constexpr int kRollTable = 64;      // entries of the plane table (a power of two)
 constexpr int kRollMaxSlots = 32;   // one producer lane per slot of a window
-constexpr int kRollXG = 4;          // planes per slot of x-major tiles (16-byte rows)
+constexpr int kRollXG = 4;          // planes per slot of x-major tiles (loaded 16 bytes a row)
 constexpr int kRollMinBlocks = 2;
-constexpr int kRollBudget2 = 110 * 1024, kRollBudget1 = 222 * 1024;  // bytes of shared memory: two CTAs per SM, one
+constexpr int kRollBudget2 = 112 * 1024, kRollBudget1 = 226 * 1024;  // bytes of shared memory: two CTAs per SM, one
 
 struct RollHdr {
     int type, tile;
     int major, dir;
-    int m0, s_len;            // the step: cells [m0, m0 + s_len) along the major axis
-    int alo, acnt, blo, bcnt; // lateral cells whose samples and taps are all staged
+    int m0, s_len;  // the step: cells [m0, m0 + s_len) along the major axis
     int pad[2];
 };
 
@@ -50,11 +59,12 @@ struct RollGeom {
     int on;      // tiles may take this major axis
     int g;       // planes per slot
     int ns;      // slots of the ring
-    int s;       // cells per step, a multiple of g
+    int s;       // cells per step
     int depth;   // steps staged ahead
     int wa, wb;  // box extents along the lateral axes A and B
-    int sb;      // floats between rows along B (along A: 1, or g for x-major)
-    int slot;    // floats per slot
+    int sb;      // floats between rows along B (along A: 1)
+    int plane;   // floats per plane
+    int slot;    // floats per slot (g planes)
 };
 
 struct RollArgs {
@@ -62,16 +72,17 @@ struct RollArgs {
     unsigned *ctr, *err;
     int ntiles, polls;
     int halo;       // cells a tap reaches beyond its sample's cell, on each side
-    int rows;       // 1: bulk copies of single rows (ragged or unaligned cube)
+    int rows;       // 1: no tensor copies (ragged or unaligned cube): bulk copies of single rows
     int goff;       // rows: floats from the 16-byte boundary below the cube to the cube
     int smem_stage; // bytes of the plane ring
+    float xbias;    // (roll_rays)
     int box_mask;   // box: entries of a ray's ring of raw samples, less one (a power of two)
     RollGeom geo[3];
 };
 
-// One tensor map per major axis (x: slots of 4 x planes; y, z: one plane).
+// The tensor maps of one plane: y-major, z-major.
 struct RollMaps {
-    CUtensorMap m[3];
+    CUtensorMap m[2];
 };
 
 struct RollShared {
@@ -79,6 +90,9 @@ struct RollShared {
     uint64_t full[kRollBars], empty[kRollBars];
     int pb[kRollTable];                   // plane q: stage index of its element (a, b) = (0, 0)
     int oa[kRollTable], ob[kRollTable];   // slot c: origin of its box
+    // cell c of a step: the lateral cells [x, x + y) along A and [z, z + w) along B whose
+    // corners and taps the planes of its window all hold
+    int4 range[kRollTable];
     int quit;
     int pad[3];
 };
@@ -88,12 +102,13 @@ template <int M>
 struct RollAxes {
     static constexpr int A = M == 0 ? 1 : 0;
     static constexpr int B = M == 2 ? 1 : 2;
-    static constexpr int SA = M == 0 ? kRollXG : 1;  // floats between neighbours along A
 };
 
 // The major axis: the one the tile's rays advance along fastest, so that lateral slopes stay
-// near 1 and the footprint of a plane small.
-__host__ __device__ __forceinline__ TileRays roll_rays(const shw_camera &c, int px0, int py0, const int on[3])
+// small and the footprint of a plane with them; x only when it is `xbias` times faster than
+// the others.
+__host__ __device__ __forceinline__ TileRays roll_rays(const shw_camera &c, int px0, int py0, const int on[3],
+                                                       float xbias)
 {
     TileRays t;
     for (int i = 0; i < 4; ++i)
@@ -102,9 +117,9 @@ __host__ __device__ __forceinline__ TileRays roll_rays(const shw_camera &c, int 
     t.major = 2;
     t.dir = 1;
     for (int k = 0; k < 3; ++k) {
-        const float s = t.u[0][k] + t.u[1][k] + t.u[2][k] + t.u[3][k];
-        if (on[k] && fabsf(s) > best) {
-            best = fabsf(s);
+        const float s = t.u[0][k] + t.u[1][k] + t.u[2][k] + t.u[3][k], f = fabsf(s) / (k == 0 ? xbias : 1.0f);
+        if (on[k] && f > best) {
+            best = f;
             t.major = k;
             t.dir = s > 0.0f ? 1 : -1;
         }
@@ -224,6 +239,47 @@ __device__ __forceinline__ void roll_row(const RollArgs &ra, float *stage, long 
     if (wrote) fence_proxy_async();  // a later bulk copy writes the same bytes
 }
 
+// Planes q0 .. q0+3 of an x-major tile: every (y, z) row of the box holds four consecutive x,
+// loaded together by one lane and written to the four planes.
+__device__ __forceinline__ void roll_xplanes(const RollArgs &ra, const RollGeom &G, float *slot, const int n[3], int q0,
+                                             int y0, int z0)
+{
+    constexpr int U = 8;  // loads in flight per lane
+    const int lane = threadIdx.x & 31;
+    const int wa = min(G.wa, n[1] - y0), total = wa * min(G.wb, n[2] - z0);
+    const float inv = 1.0f / (float)wa;
+    for (int i0 = lane; i0 < total; i0 += 32 * U) {
+        float4 v[U];
+        int at[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int i = i0 + 32 * u;
+            at[u] = -1;
+            if (i < total) {
+                const int b = (int)(((float)i + 0.5f) * inv), a = i - b * wa;  // (exact: i < 2^16)
+                at[u] = b * G.sb + a;
+                const float *p = ra.cube + ((size_t)(z0 + b) * n[1] + (y0 + a)) * n[0] + q0;
+                if (!ra.rows) {
+                    v[u] = __ldg(reinterpret_cast<const float4 *>(p));
+                } else {
+                    v[u].x = __ldg(p);
+                    v[u].y = q0 + 1 < n[0] ? __ldg(p + 1) : 0.0f;
+                    v[u].z = q0 + 2 < n[0] ? __ldg(p + 2) : 0.0f;
+                    v[u].w = q0 + 3 < n[0] ? __ldg(p + 3) : 0.0f;
+                }
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (at[u] >= 0) {
+                slot[at[u]] = v[u].x;
+                slot[at[u] + G.plane] = v[u].y;
+                slot[at[u] + 2 * G.plane] = v[u].z;
+                slot[at[u] + 3 * G.plane] = v[u].w;
+            }
+    }
+}
+
 template <int M>
 __device__ __forceinline__ bool roll_produce(const TileRays &r, bool persp, const CUtensorMap *map,
                                              const RenderArgs &a, const RollArgs &ra, int tile, float *stage,
@@ -286,25 +342,28 @@ __device__ __forceinline__ bool roll_produce(const TileRays &r, bool persp, cons
             ob = min(max(lo, 0), n_b - 1);
             sh.oa[c & (kRollTable - 1)] = oa;
             sh.ob[c & (kRollTable - 1)] = ob;
-            int pb = (c % G.ns) * G.slot - oa * AX::SA - ob * G.sb;
+            int pb = (c % G.ns) * G.slot - oa - ob * G.sb;
             if (M != 0 && ra.rows) {
                 // equal global and shared addresses modulo 16 bytes (the row pitch agrees already)
                 const int want = ra.goff + (M == 2 ? (c * n[1] & 3) * (n[0] & 3) : (c & 3) * (n[0] & 3));
                 pb += 4 + ((want - pb) & 3);
             }
 #pragma unroll
-            for (int j = 0; j < g; ++j) sh.pb[(q0 + j) & (kRollTable - 1)] = pb + j;
+            for (int j = 0; j < g; ++j) sh.pb[(q0 + j) & (kRollTable - 1)] = pb + j * G.plane;
         }
         __syncwarp();
-        if (M == 0 || !ra.rows) {
+        if constexpr (M == 0) {
+            for (int c = c0; c <= c1; ++c)
+                roll_xplanes(ra, G, stage + (c % G.ns) * G.slot, n, c * g, sh.oa[c & (kRollTable - 1)],
+                             sh.ob[c & (kRollTable - 1)]);
+            fence_proxy_async();  // a later copy may write the same bytes
+        } else if (!ra.rows) {
             if (lane < cnt) {
                 const int c = c0 + lane;
                 float *dst = stage + (size_t)(c % G.ns) * G.slot;
                 if (tma_dst_ok(dst, ra.err)) {  // always: slots are 128-byte multiples
-                    mbar_expect_tx(bar, (uint32_t)(G.wa * G.wb * g * 4));
-                    if constexpr (M == 0)
-                        tma_load_3d(dst, map, c * g, oa, ob, bar);
-                    else if constexpr (M == 1)
+                    mbar_expect_tx(bar, (uint32_t)(G.wa * G.wb * 4));
+                    if constexpr (M == 1)
                         tma_load_3d(dst, map, oa, c, ob, bar);
                     else
                         tma_load_3d(dst, map, oa, ob, c, bar);
@@ -320,21 +379,21 @@ __device__ __forceinline__ bool roll_produce(const TileRays &r, bool persp, cons
                 roll_row(ra, stage, nvox, row, x, min(G.wa, n_a - x), sh.pb[ci] + b * G.sb + x, bar);
             }
         }
-        // the lateral cells whose samples and taps every plane of the window holds
-        int alo = -1, ahi = n_a - 1, blo = -1, bhi = n_b - 1;
-        if (slo + lane <= shi) {
-            const int c = slo + lane, ci = c & (kRollTable - 1), q0 = c * g;
-            const bool own = q0 + g - 1 >= m0 && q0 <= m0 + s;  // planes of the step's own cells
-            const int h = own ? H : 0, x = sh.oa[ci], y = sh.ob[ci];
-            if (x > 0) alo = x + h;
-            if (x + G.wa < n_a) ahi = x + G.wa - 2 - h;
-            if (y > 0) blo = y + h;
-            if (y + G.wb < n_b) bhi = y + G.wb - 2 - h;
+        if (lane < s) {
+            const int cell = m0 + lane;
+            const int w0 = max(cell - H, 0) / g, w1 = min(cell + 1 + H, n_m - 1) / g;
+            int alo = -1, ahi = n_a - 1, blo = -1, bhi = n_b - 1;
+            for (int c = w0; c <= w1; ++c) {
+                const int ci = c & (kRollTable - 1), q0 = c * g;
+                const bool own = q0 + g - 1 >= cell && q0 <= cell + 1;  // holds the cell's own planes
+                const int h = own ? H : 0, x = sh.oa[ci], y = sh.ob[ci];
+                if (x > 0) alo = max(alo, x + h);
+                if (x + G.wa < n_a) ahi = min(ahi, x + G.wa - 2 - h);
+                if (y > 0) blo = max(blo, y + h);
+                if (y + G.wb < n_b) bhi = min(bhi, y + G.wb - 2 - h);
+            }
+            sh.range[cell & (kRollTable - 1)] = make_int4(alo, max(ahi - alo + 1, 0), blo, max(bhi - blo + 1, 0));
         }
-        alo = __reduce_max_sync(0xffffffffu, alo);
-        ahi = __reduce_min_sync(0xffffffffu, ahi);
-        blo = __reduce_max_sync(0xffffffffu, blo);
-        bhi = __reduce_min_sync(0xffffffffu, bhi);
         if (lane == 0) {
             RollHdr h;
             h.type = kStageSlab;
@@ -343,10 +402,6 @@ __device__ __forceinline__ bool roll_produce(const TileRays &r, bool persp, cons
             h.dir = dir;
             h.m0 = m0;
             h.s_len = s;
-            h.alo = alo;
-            h.acnt = max(ahi - alo + 1, 0);
-            h.blo = blo;
-            h.bcnt = max(bhi - blo + 1, 0);
             sh.hdr[st] = h;
         }
         __syncwarp();  // every lane's expected bytes and table entries come before the arrival
@@ -377,14 +432,14 @@ __device__ __forceinline__ void roll_producer(const CUtensorMap *maps, const shw
         if (!ring.post_plain(kStageTile, (int)t)) break;
         int tx, ty;
         slab_tile((int)t, a, tx, ty);
-        const TileRays r = roll_rays(cam, tx * kSlabTW, ty * kSlabTH, on);
+        const TileRays r = roll_rays(cam, tx * kSlabTW, ty * kSlabTH, on, ra.xbias);
         const bool persp = !cam.ortho;
         if (r.major == 0)
-            ok = roll_produce<0>(r, persp, &maps[0], a, ra, (int)t, stage, ring);
+            ok = roll_produce<0>(r, persp, nullptr, a, ra, (int)t, stage, ring);
         else if (r.major == 1)
-            ok = roll_produce<1>(r, persp, &maps[1], a, ra, (int)t, stage, ring);
+            ok = roll_produce<1>(r, persp, &maps[0], a, ra, (int)t, stage, ring);
         else
-            ok = roll_produce<2>(r, persp, &maps[2], a, ra, (int)t, stage, ring);
+            ok = roll_produce<2>(r, persp, &maps[1], a, ra, (int)t, stage, ring);
         if (ok) ok = ring.post_plain(kStageTileEnd, (int)t);
     }
     // no exit while a copy into this CTA's shared memory is in flight: wait (bounded) for the
@@ -419,7 +474,7 @@ __device__ __forceinline__ float roll_value(const float *stage, const int *pbt, 
                                             const long long P[3], const RenderArgs &a)
 {
     using AX = RollAxes<M>;
-    constexpr int A = AX::A, B = AX::B, SA = AX::SA;
+    constexpr int A = AX::A, B = AX::B;
     int i0[3], i1[3];
     float f[3];
 #pragma unroll
@@ -449,7 +504,7 @@ __device__ __forceinline__ float roll_value(const float *stage, const int *pbt, 
         return trilerp(c, fx, fy, fz);
     };
     const int m0 = plane(i0[M]), m1 = plane(i1[M]);
-    const int a0 = i0[A] * SA, a1 = CLAMP ? i1[A] * SA : a0 + SA;
+    const int a0 = i0[A], a1 = CLAMP ? i1[A] : a0 + 1;
     const int b0 = i0[B] * sb, b1 = CLAMP ? i1[B] * sb : b0 + sb;
     float v = fetch8(m0, m1, a0, a1, b0, b1, f[0], f[1], f[2]);
     if constexpr (TAPS) {
@@ -469,8 +524,7 @@ __device__ __forceinline__ float roll_value(const float *stage, const int *pbt, 
                         t = fetch8(plane(t0), plane(t1), a0, a1, b0, b1, M == 0 ? tf : f[0], M == 1 ? tf : f[1],
                                    M == 2 ? tf : f[2]);
                     } else if (ax == A) {
-                        const int u0 = t0 * SA, u1 = CLAMP ? t1 * SA : u0 + SA;
-                        t = fetch8(m0, m1, u0, u1, b0, b1, A == 0 ? tf : f[0], A == 1 ? tf : f[1], f[2]);
+                        t = fetch8(m0, m1, t0, CLAMP ? t1 : t0 + 1, b0, b1, A == 0 ? tf : f[0], A == 1 ? tf : f[1], f[2]);
                     } else {
                         const int u0 = t0 * sb, u1 = CLAMP ? t1 * sb : u0 + sb;
                         t = fetch8(m0, m1, a0, a1, u0, u1, f[0], B == 1 ? tf : f[1], B == 2 ? tf : f[2]);
@@ -552,26 +606,41 @@ struct RollMarch {
 template <int M, int MODE, int KIND, class S>
 __device__ __forceinline__ bool roll_step(const S &s, const RenderArgs &a, RollMarch<MODE, KIND> &q, long long DX,
                                           long long DY, long long DZ, const RollHdr &h, const float *stage,
-                                          const int *pbt, int sb, int lim, float *ring, int mask)
+                                          const RollShared &sh, int sb, int lim, float *ring, int mask)
 {
     using AX = RollAxes<M>;
+    constexpr bool TAPS = KIND == kRollTaps;
     const int n[3] = {s.nx, s.ny, s.nz};
-    const int m_edge = h.dir > 0 ? h.m0 : h.m0 + h.s_len - 1;
-    while (q.k < q.kend) {
+    for (;;) {
+        // samples that need no clamping, as long as the step holds them
+        const int kin = min(q.kb, q.kend);
+        while (q.k >= q.ka && q.k < kin) {
+            const long long P[3] = {q.X, q.Y, q.Z};
+            const int cm = fx_cell(P[M]);
+            if ((unsigned)(cm - h.m0) >= (unsigned)h.s_len) break;
+            const int4 in = sh.range[cm & (kRollTable - 1)];
+            if ((unsigned)(fx_cell(P[AX::A]) - in.x) >= (unsigned)in.y ||
+                (unsigned)(fx_cell(P[AX::B]) - in.z) >= (unsigned)in.w)
+                break;
+            const bool stop = q.take(a, roll_value<M, false, TAPS>(stage, sh.pb, sb, lim, n, P, a), ring, mask);
+            q.X += DX;
+            q.Y += DY;
+            q.Z += DZ;
+            ++q.k;
+            if (stop) return true;
+        }
+        if (q.k >= q.kend) return false;
+        // one sample at the cube's faces, outside the staged boxes, or of a later step
         const long long P[3] = {q.X, q.Y, q.Z};
-        const int cm = clampi(fx_cell(P[M]), -1, n[M] - 1);
-        const int rel = h.dir > 0 ? cm - m_edge : m_edge - cm;
+        const int cm = clampi(fx_cell(P[M]), -1, n[M] - 1), rel = h.dir > 0 ? cm - h.m0 : h.m0 + h.s_len - 1 - cm;
         if (rel >= h.s_len) return false;  // a later step's
         const int ca = clampi(fx_cell(P[AX::A]), -1, n[AX::A] - 1), cb = clampi(fx_cell(P[AX::B]), -1, n[AX::B] - 1);
+        const int4 in = sh.range[cm & (kRollTable - 1)];
         float v;
-        if (rel >= 0 && (unsigned)(ca - h.alo) < (unsigned)h.acnt && (unsigned)(cb - h.blo) < (unsigned)h.bcnt) {
-            if (q.k >= q.ka && q.k < q.kb)
-                v = roll_value<M, false, KIND == kRollTaps>(stage, pbt, sb, lim, n, P, a);
-            else
-                v = roll_value<M, true, KIND == kRollTaps>(stage, pbt, sb, lim, n, P, a);
-        } else {
-            v = roll_global<KIND == kRollTaps>(s, q.X, q.Y, q.Z, a);
-        }
+        if (rel >= 0 && (unsigned)(ca - in.x) < (unsigned)in.y && (unsigned)(cb - in.z) < (unsigned)in.w)
+            v = roll_value<M, true, TAPS>(stage, sh.pb, sb, lim, n, P, a);
+        else
+            v = roll_global<TAPS>(s, q.X, q.Y, q.Z, a);
         const bool stop = q.take(a, v, ring, mask);
         q.X += DX;
         q.Y += DY;
@@ -579,7 +648,6 @@ __device__ __forceinline__ bool roll_step(const S &s, const RenderArgs &a, RollM
         ++q.k;
         if (stop) return true;
     }
-    return false;
 }
 
 template <int MODE, int KIND, class S>
@@ -631,13 +699,13 @@ __device__ __forceinline__ void roll_consumer(const S &s, const shw_camera &cam,
             if (live) {
                 bool stop;
                 if (h.major == 0)
-                    stop = roll_step<0, MODE, KIND>(s, a, q, r.D[0], r.D[1], r.D[2], h, stage, sh.pb, ra.geo[0].sb,
+                    stop = roll_step<0, MODE, KIND>(s, a, q, r.D[0], r.D[1], r.D[2], h, stage, sh, ra.geo[0].sb,
                                                     ra.smem_stage / 4, ring, ra.box_mask);
                 else if (h.major == 1)
-                    stop = roll_step<1, MODE, KIND>(s, a, q, r.D[0], r.D[1], r.D[2], h, stage, sh.pb, ra.geo[1].sb,
+                    stop = roll_step<1, MODE, KIND>(s, a, q, r.D[0], r.D[1], r.D[2], h, stage, sh, ra.geo[1].sb,
                                                     ra.smem_stage / 4, ring, ra.box_mask);
                 else
-                    stop = roll_step<2, MODE, KIND>(s, a, q, r.D[0], r.D[1], r.D[2], h, stage, sh.pb, ra.geo[2].sb,
+                    stop = roll_step<2, MODE, KIND>(s, a, q, r.D[0], r.D[1], r.D[2], h, stage, sh, ra.geo[2].sb,
                                                     ra.smem_stage / 4, ring, ra.box_mask);
                 if (stop) live = false;
             }
@@ -708,8 +776,43 @@ inline void roll_extent(const TileRays &r, const int n[3], int H, int g, int &wa
     }
 }
 
-// Slots a step's window spans, with `depth` steps staged ahead.
-inline int roll_slots(int H, int s, int g, int depth) { return (H + g - 1) / g + (s + H) / g + 1 + depth * s / g; }
+// Slots that the windows of a step and of the `depth` steps staged ahead of it span, for the
+// step start that spans most (steps start at multiples of s, slots at multiples of g).
+inline int roll_slots(int H, int s, int g, int depth)
+{
+    const int back = (H + g - 1) / g + 1;  // (keeps the divisions below on positive numbers)
+    int most = 0;
+    for (int m = 0; m < s * g; m += s)
+        most = std::max(most, (m + s + H + depth * s + back * g) / g - (m - H + back * g) / g + 1);
+    return most;
+}
+
+// Lateral extent along A of a warp's 8 x 4 pixels where their rays cross one plane (the
+// centre tile, at the cube's centre).
+template <int M>
+inline float roll_warp_extent(const TileRays &r, const int n[3])
+{
+    TileLines<M> L;
+    if (!tile_lines<M>(r, L)) return 8.0f;
+    const float m = 0.5f * (float)(n[M] - 1);
+    float p[4];
+    for (int i = 0; i < 4; ++i) p[i] = L.B[i][RollAxes<M>::A] * m + L.A[i][RollAxes<M>::A];
+    return fabsf(p[1] - p[0]) * (7.0f / (kSlabTW - 1)) + fabsf(p[2] - p[0]) * (3.0f / (kSlabTH - 1));
+}
+
+// The smallest row pitch >= w, congruent to `mod4` modulo 4, that puts neighbouring rows `ext`
+// banks or so apart: the rows of a warp's footprint, ext floats long, then miss each other.
+inline int roll_pitch(int w, float ext, int mod4)
+{
+    auto ok = [&](int p) {
+        const int q = (p - mod4) & 31;
+        if (ext <= 4.0f) return (q & 7) == 4;
+        if (ext <= 8.0f) return (q & 15) == 8;
+        return q == 12 || q == 16 || q == 20;
+    };
+    while (!ok(w)) ++w;
+    return w;
+}
 
 // The launch's staging geometry: for each major axis that its tiles take, box extents that
 // hold the sampled tiles' footprints, the longest step whose window fits the shared memory
@@ -717,55 +820,49 @@ inline int roll_slots(int H, int s, int g, int depth) { return (H + g - 1) / g +
 inline bool roll_geometry(const shw_camera &cam, const int n[3], int H, bool tmaps, int budget, int smax, int min_s,
                           RollArgs &ra)
 {
-    const int on[3] = {tmaps, 1, 1};
+    const int on[3] = {1, 1, 1};
     int wa[3] = {0, 0, 0}, wb[3] = {0, 0, 0};
-    bool used[3] = {false, false, false};
+    float ext[3] = {8.0f, 8.0f, 8.0f};
     const int tx = ceil_div(cam.width, kSlabTW), ty = ceil_div(cam.height, kSlabTH);
     for (int j = 0; j < 5; ++j)
         for (int i = 0; i < 5; ++i) {
             const TileRays r = roll_rays(cam, (int)((long long)(tx - 1) * i / 4) * kSlabTW,
-                                         (int)((long long)(ty - 1) * j / 4) * kSlabTH, on);
-            used[r.major] = true;
-            if (r.major == 0) roll_extent<0>(r, n, H, kRollXG, wa[0], wb[0]);
-            else if (r.major == 1) roll_extent<1>(r, n, H, 1, wa[1], wb[1]);
-            else roll_extent<2>(r, n, H, 1, wa[2], wb[2]);
+                                         (int)((long long)(ty - 1) * j / 4) * kSlabTH, on, ra.xbias);
+            const int M = r.major, g = M == 0 ? kRollXG : 1;
+            const float was = M == 0   ? (roll_extent<0>(r, n, H, g, wa[0], wb[0]), roll_warp_extent<0>(r, n))
+                              : M == 1 ? (roll_extent<1>(r, n, H, g, wa[1], wb[1]), roll_warp_extent<1>(r, n))
+                                       : (roll_extent<2>(r, n, H, g, wa[2], wb[2]), roll_warp_extent<2>(r, n));
+            if (ext[M] == 8.0f || (i == 2 && j == 2)) ext[M] = was;
         }
     int stage = 0;
     bool any = false;
     for (int M = 0; M < 3; ++M) {
         RollGeom &G = ra.geo[M];
         G = RollGeom{};
-        if (!used[M] || wa[M] <= 0 || wb[M] <= 0) {
-            // no sampled tile: a tile that takes this axis all the same reads global memory
-            continue;
-        }
+        if (wa[M] <= 0 || wb[M] <= 0) continue;  // no sampled tile takes this axis: none will
         const int A = M == 0 ? 1 : 0, B = M == 2 ? 1 : 2;
         G.g = M == 0 ? kRollXG : 1;
-        G.wb = std::min(wb[M] + 1, n[B]);
-        G.wa = std::min(wa[M] + 1, n[A]);
-        if (M == 0) {
-            G.wa |= 1;  // an odd number of 16-byte rows: neighbours along B on other banks
-            G.sb = G.g * G.wa;
-            G.slot = G.sb * G.wb;
-        } else if (tmaps) {
-            G.wa = (G.wa + 3 + 3) / 4 * 4;      // the box starts on 16 bytes
-            if (G.wa % 8 == 0) G.wa += 4;       // an odd number of 16 bytes per row
-            G.sb = G.wa;
-            G.slot = G.sb * G.wb;
+        // room for the tiles and planes between the sampled ones
+        G.wb = std::min(wb[M] + 2 + (wb[M] - 2 * H) / 10, n[B]);
+        G.wa = std::min(wa[M] + 2 + (wa[M] - 2 * H) / 10, n[A]);
+        int pad = 0;
+        if (M != 0 && tmaps) {
+            G.sb = G.wa = roll_pitch(G.wa + 3, ext[M], 0);  // a tensor copy's rows; its x start on 16 bytes
+        } else if (M != 0) {
+            G.sb = roll_pitch(G.wa + 6, ext[M], (M == 2 ? n[0] : (n[0] & 3) * (n[1] & 3)) & 3);
+            pad = 16;
         } else {
-            const int want = (M == 2 ? n[0] : (n[0] & 3) * (n[1] & 3)) & 3;  // row pitch of the cube modulo 4
-            G.sb = G.wa + 6;
-            G.sb += (want - G.sb) & 3;
-            G.slot = G.sb * G.wb + 16;
+            G.sb = roll_pitch(G.wa, ext[M], 0);
         }
         if (G.wa > 256 || G.wb > 256) return false;
-        G.slot = (G.slot + 31) & ~31;
+        G.plane = (G.sb * G.wb + pad + 31) & ~31;
+        G.slot = G.plane * G.g;
         G.depth = 1;
         const int cap = std::min(std::min(kRollMaxSlots, kRollTable / G.g), budget / (G.slot * 4));
         G.s = 0;
-        for (int s = G.g; s <= std::max(smax, G.g); s += G.g)
+        for (int s = 1; s <= smax; ++s)
             if (roll_slots(H, s, G.g, G.depth) <= cap) G.s = s;
-        if (G.s < std::max(min_s, G.g)) return false;
+        if (G.s < min_s) return false;
         G.ns = roll_slots(H, G.s, G.g, G.depth);
         G.on = 1;
         any = true;
@@ -784,7 +881,7 @@ shw_status roll_launch_one(const RollMaps &maps, const S &s, const shw_camera &c
         cudaGetLastError();
         return SHW_ECUDA;
     }
-    const int nsm = sm_count(), per_sm = smem <= (size_t)113 * 1024 ? 2 : 1;
+    const int nsm = sm_count(), per_sm = smem <= (size_t)kRollBudget2 ? 2 : 1;
     if (nsm <= 0) return SHW_ECUDA;
     const long long grid = std::min<long long>((long long)per_sm * nsm, ra.ntiles);
     kern<<<(unsigned)std::max<long long>(grid, 1), kSlabThreads, smem, st>>>(maps, s, cam, a, ra);
@@ -817,6 +914,10 @@ shw_status roll_launch(int mode, const shw_volume &v, const shw_camera &cam, con
         ra.box_mask = len - 1;
         extra += (size_t)len * 32 * kSlabWarps * 4;
     }
+    // Taps: the true major axis (the planes hold the taps' reach on both sides, and only small
+    // slopes keep two CTAs on an SM).  The box: x-major planes cost the producer a transposition,
+    // so steep y- and z-major ones are taken up to a slope of 3.
+    ra.xbias = KIND == kRollTaps ? 1.0f : 3.0f;
     // two CTAs per SM where a step of at least two cells fits, else one
     const int smax = KIND == kRollTaps ? 4 : 12;
     if (!roll_geometry(cam, n, ra.halo, tmaps, kRollBudget2 - (int)extra, smax, 2, ra) &&
@@ -825,9 +926,8 @@ shw_status roll_launch(int mode, const shw_volume &v, const shw_camera &cam, con
     RollMaps maps{};
     if (tmaps) {
         const RollGeom *G = ra.geo;
-        if ((G[0].on && !encode_tmap_3d(&maps.m[0], s.v, 4, v.nx, v.ny, v.nz, kRollXG, G[0].wa, G[0].wb)) ||
-            (G[1].on && !encode_tmap_3d(&maps.m[1], s.v, 4, v.nx, v.ny, v.nz, G[1].wa, 1, G[1].wb)) ||
-            (G[2].on && !encode_tmap_3d(&maps.m[2], s.v, 4, v.nx, v.ny, v.nz, G[2].wa, G[2].wb, 1)))
+        if ((G[1].on && !encode_tmap_3d(&maps.m[0], s.v, 4, v.nx, v.ny, v.nz, G[1].wa, 1, G[1].wb)) ||
+            (G[2].on && !encode_tmap_3d(&maps.m[1], s.v, 4, v.nx, v.ny, v.nz, G[2].wa, G[2].wb, 1)))
             return SHW_EUNSUPPORTED;
     }
     RenderArgs a = a0;
