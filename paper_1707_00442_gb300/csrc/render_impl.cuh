@@ -544,7 +544,12 @@ __device__ __forceinline__ bool march(const S &s, const S &s2, const RenderArgs 
                                       long long DY, long long DZ, int k0, int k1, int &kdone,
                                       const long long *U = nullptr)
 {
-    for (int k = k0; k < k1; ++k) {
+    // One exit only (here and in the interior loops): with a return inside the loop the lanes of
+    // a warp stayed apart after the branches around the loads (18 of 32 active in compositing;
+    // a 750 x 750 x 70 cube on 1000 x 1000: 830 us with it, 446 us without).
+    bool stop = false;
+    int k = k0;
+    for (; k < k1 && !stop; ++k) {
         if constexpr (MODE == SHW_RATIO_MIP) {
             // Algorithm 13: each cube's maximum; a NaN sample counts as DATAMIN
             float r1, r2;
@@ -564,17 +569,14 @@ __device__ __forceinline__ bool march(const S &s, const S &s2, const RenderArgs 
                 v = filter_value(isnan(v) ? a.lo : v, a);
             }
             v = isnan(v) ? a.lo : v;  // a NaN sample counts as DATAMIN
-            if (st.update(v, k)) {
-                kdone = k + 1;
-                return true;
-            }
+            stop = st.update(v, k);
         }
         X += DX;
         Y += DY;
         Z += DZ;
     }
-    kdone = k1;
-    return false;
+    kdone = max(k, k0);
+    return stop;
 }
 
 #ifndef SHW_PREFETCH
@@ -599,7 +601,9 @@ __device__ __forceinline__ bool march_interior_pair(const S &s, const RenderArgs
     int cx = fx_cell(X), cy = fx_cell(Y), cz = fx_cell(Z);
     float2 cur[8];
     s.template corners2<false>(cx, cy, cz, cur);
-    for (int k = k0; k < k1; ++k) {
+    bool stop = false;
+    int k = k0;
+    for (; k < k1 && !stop; ++k) {
         const long long Xn = X + DX, Yn = Y + DY, Zn = Z + DZ;
         const int nx = fx_cell(Xn), ny = fx_cell(Yn), nz = fx_cell(Zn);
         const bool pf = ((nx != cx) | (ny != cy) | (nz != cz)) && k + 1 < k1;
@@ -613,10 +617,7 @@ __device__ __forceinline__ bool march_interior_pair(const S &s, const RenderArgs
             // Algorithm 14: ratio where cube1 exceeds the floor, else DATAMIN
             float v = (c1 > a.ratio_floor) ? __fdiv_rn(c2, c1) : a.lo;
             v = isnan(v) ? a.lo : v;
-            if (st.update(v, k)) {
-                kdone = k + 1;
-                return true;
-            }
+            stop = st.update(v, k);
         }
         if (pf) {
 #pragma unroll
@@ -629,8 +630,8 @@ __device__ __forceinline__ bool march_interior_pair(const S &s, const RenderArgs
         Y = Yn;
         Z = Zn;
     }
-    kdone = k1;
-    return false;
+    kdone = k;
+    return stop;
 }
 
 // march_interior_single: one or two separate cubes.
@@ -648,7 +649,9 @@ __device__ __forceinline__ bool march_interior_single(const S &s, const S &s2, c
     float cur[8], cur2[8];
     s.template corners<false>(cx, cy, cz, cur);
     if constexpr (TWO) s2.template corners<false>(cx, cy, cz, cur2);
-    for (int k = k0; k < k1; ++k) {
+    bool stop = false;
+    int k = k0;
+    for (; k < k1 && !stop; ++k) {
         const long long Xn = X + DX, Yn = Y + DY, Zn = Z + DZ;
         const int nx = fx_cell(Xn), ny = fx_cell(Yn), nz = fx_cell(Zn);
         const bool change = (nx != cx) | (ny != cy) | (nz != cz);
@@ -673,10 +676,7 @@ __device__ __forceinline__ bool march_interior_single(const S &s, const S &s2, c
         }
         if constexpr (MODE != SHW_RATIO_MIP) {
             v = isnan(v) ? a.lo : v;  // a NaN sample counts as DATAMIN
-            if (st.update(v, k)) {
-                kdone = k + 1;
-                return true;
-            }
+            stop = st.update(v, k);
         }
         if (pf) {
 #pragma unroll
@@ -692,8 +692,8 @@ __device__ __forceinline__ bool march_interior_single(const S &s, const S &s2, c
         Y = Yn;
         Z = Zn;
     }
-    kdone = k1;
-    return false;
+    kdone = k;
+    return stop;
 }
 
 // The interior loop for the sampler at hand.
