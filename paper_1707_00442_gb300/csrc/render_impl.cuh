@@ -893,11 +893,20 @@ int sm_count();
 // Persistent form: every warp takes the next warp tile (centre-out order, as above)
 // from a global counter until none is left, so no SM idles while rays of very
 // different lengths finish and no CTA launch overhead is paid per tile.
-#ifndef SHW_RENDER_MINB
-#define SHW_RENDER_MINB 1  // minimum resident CTAs per SM the persistent kernel is compiled for
-#endif
+//
+// Resident CTAs per SM the kernel is compiled for.  It waits on its gathers, so warps in flight
+// count for more than registers: with 8 (the registers the set-up would take) 512^3 nearest on
+// 1000 x 1000 takes 861 us, with 12 709 us, 16 740; compositing 750 x 750 x 70 448 / 336 / 345; the
+// ratio of two cubes, which holds 32 corners, 240 us with 8, 206 with 10, 213 with 12, 373 with
+// 16 (spills).  In-ray smoothing keeps what the compiler takes.
+template <int MODE, int INTERP, int SMK>
+constexpr int render_min_ctas()
+{
+    if (SMK > 0) return 1;
+    return INTERP == SHW_TRILINEAR && two_cubes<MODE> ? 10 : 12;
+}
 template <int MODE, int INTERP, class S, int SMK = 0>
-__global__ void __launch_bounds__(kRenderThreads, SHW_RENDER_MINB)
+__global__ void __launch_bounds__(kRenderThreads, (render_min_ctas<MODE, INTERP, SMK>()))
     render_kernel_persistent(S s, S s2, shw_camera cam, RenderArgs a, unsigned *ctr, int nwarp_tiles)
 {
     const int lane = threadIdx.x & 31;
@@ -975,9 +984,14 @@ shw_status launch_render_modes(int mode, int interp, const S &s, const S &s2, co
     unsigned *ctr = SHW_RENDER_PERSISTENT ? work_counter(st) : nullptr;
     const int nsm = sm_count();
     const int nwarp_tiles = (int)(tiles * kCtaWarps);
-    // persistent grid: as many CTAs as fit on the device at once (at most one per tile)
+    // persistent grid: as many CTAs as fit on the device at once (at most one per tile).  An
+    // image of only a few tiles per CTA takes fewer CTAs, down to 8 per SM: more would leave
+    // nothing to even out the long rays with (128^3 on 500 x 500, compositing: 137 us with 8 per
+    // SM, 193 with 12; 1000 x 1000: 389 and 383).  Nearest sampling's rays are too short to
+    // mind (45 us with 11 per SM, 53 with 8).
     auto persistent = [&](auto kern, int per_sm) {
-        const long long g = std::min<long long>((long long)per_sm * nsm, tiles);
+        long long g = std::min<long long>((long long)per_sm * nsm, tiles);
+        if (SMK == 0 && interp != SHW_NEAREST) g = std::min(g, std::max(tiles / 4, 8LL * nsm));
         kern<<<(unsigned)std::max<long long>(g, 1), block, 0, st>>>(s, s2, cam, a, ctr, nwarp_tiles);
     };
     if (SMK > 0 && (ctr == nullptr || nsm <= 0)) return SHW_ECUDA;
