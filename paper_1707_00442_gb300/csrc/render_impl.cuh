@@ -894,16 +894,19 @@ int sm_count();
 // from a global counter until none is left, so no SM idles while rays of very
 // different lengths finish and no CTA launch overhead is paid per tile.
 //
-// Resident CTAs per SM the kernel is compiled for.  It waits on its gathers, so warps in flight
-// count for more than registers: with 8 (the registers the set-up would take) 512^3 nearest on
-// 1000 x 1000 takes 861 us, with 12 709 us, 16 740; compositing 750 x 750 x 70 448 / 336 / 345; the
-// ratio of two cubes, which holds 32 corners, 240 us with 8, 206 with 10, 213 with 12, 373 with
-// 16 (spills).  In-ray smoothing keeps what the compiler takes.
+// Resident CTAs per SM the kernel is compiled for (1: what the compiler takes, 8 for most, from
+// the registers of the ray set-up).  It waits on its gathers, so where the march itself needs
+// few registers more warps in flight win: nearest sampling of 512^3 on 1000 x 1000 861 us with
+// 11, 709 with 12 (80 registers; 16: 740), compositing 750 x 750 x 70 448 / 336 / 345 with
+// 8 / 12 / 16, the ratio of two cubes, which holds 32 corners, 240 / 206 / 213 / 373 with
+// 8 / 10 / 12 / 16 (spills).  The other trilinear modes gain nothing and lose where neighbouring
+// rays share their loads (395 x 395 x 41 along z: 172 us with 8, 208 with 12).
 template <int MODE, int INTERP, int SMK>
 constexpr int render_min_ctas()
 {
     if (SMK > 0) return 1;
-    return INTERP == SHW_TRILINEAR && two_cubes<MODE> ? 10 : 12;
+    if (INTERP == SHW_NEAREST || is_composite<MODE>) return 12;
+    return two_cubes<MODE> ? 10 : 1;
 }
 template <int MODE, int INTERP, class S, int SMK = 0>
 __global__ void __launch_bounds__(kRenderThreads, (render_min_ctas<MODE, INTERP, SMK>()))

@@ -16,11 +16,15 @@ shw_status render_slab(int mode, int interp, const shw_volume &v, const shw_came
     switch (v.storage) {
     case SHW_F32: {
         if (ratio || v.nx % 4 != 0) return SHW_EUNSUPPORTED;  // (the ratio of two separate cubes)
+        if (!debug(SHW_DEBUG_REQUIRE_STAGING) && !slab_pays<SlabGeom<ElemF32>>(cam, v.nx, v.ny, v.nz))
+            return SHW_EUNSUPPORTED;
         const SamplerF32<int> s{static_cast<const float *>(v.data), v.nx, v.ny, v.nz, v.nx, v.nx * v.ny};
         return slab_launch<ElemF32>(mode, s, v.data, cam, a, st);
     }
     case SHW_F32_PAIR: {
         if (!ratio || v.nx % 2 != 0) return SHW_EUNSUPPORTED;
+        if (!debug(SHW_DEBUG_REQUIRE_STAGING) && !slab_pays<SlabGeom<ElemF32Pair>>(cam, v.nx, v.ny, v.nz))
+            return SHW_EUNSUPPORTED;
         const SamplerF32Pair<int> s{static_cast<const float2 *>(v.data), v.nx, v.ny, v.nz, v.nx, v.nx * v.ny};
         return slab_launch<ElemF32Pair>(mode, s, v.data, cam, a, st);
     }

@@ -138,7 +138,7 @@ struct TileRays {
     int major, dir;
 };
 
-__device__ __forceinline__ TileRays tile_rays(const shw_camera &c, int px0, int py0)
+__host__ __device__ __forceinline__ TileRays tile_rays(const shw_camera &c, int px0, int py0)
 {
     TileRays t;
 #pragma unroll
@@ -733,6 +733,61 @@ shw_status slab_launch_one(const SlabMaps &maps, const S &s, const shw_camera &c
     const long long grid = std::min<long long>((long long)per_sm * nsm, sa.ntiles);
     kern<<<(unsigned)std::max<long long>(grid, 1), kSlabThreads, kSlabSmemBytes, st>>>(maps, s, cam, a, sa);
     return after_launch();
+}
+
+// Whether staging pays for a float32 cube or pair storage (the gather marcher is the
+// alternative), from the tile at the cube's projected centre where its rays pass its middle:
+//   - its footprint in a slab of one cell has to fit the staged box, or most samples would read
+//     global memory one at a time (300^3 on 500 x 500, yaw 70: 545 us staged, 388 gathered);
+//     x-major boxes stay below three quarters of a stage, fuller ones leave slabs of one cell
+//     (200^3 on 400 x 400, yaw 85: 344 against 180).  A cube larger than the second-level cache
+//     is gathered from HBM, and a footprint up to 50 cells wide still stages better (512^3 on
+//     640 x 640: 816 against 1298; the pair storage of 512^3 on 1000 x 1000, yaw 70: 2693
+//     against 3835);
+//   - above a fifth of a voxel per pixel: below, the gathers hit the first-level cache and the
+//     stages' hand-overs cost more (64^3 on 1000 x 1000, compositing: 267 against 217).
+// Over 700 renders (48^3 .. 512^3 and oblong cubes, 128^2 .. 1000^2, five views, MIP and
+// compositing) the rule is 2 % from the better of the two on average, always staging 21 %.
+template <class G>
+inline bool slab_pays(const shw_camera &c, int nx, int ny, int nz)
+{
+    float px, py;
+    project_centre(c, nx, ny, nz, px, py);
+    const int x0 = (int)fminf(fmaxf(px, 0.0f), (float)(c.width - 1)) / kSlabTW * kSlabTW;
+    const int y0 = (int)fminf(fmaxf(py, 0.0f), (float)(c.height - 1)) / kSlabTH * kSlabTH;
+    float pitch = 2.0f * c.ortho_half_h / (float)c.height;  // voxels per pixel at the centre
+    if (!c.ortho) {
+        const float q[3] = {0.5f * (nx - 1) - c.eye[0], 0.5f * (ny - 1) - c.eye[1], 0.5f * (nz - 1) - c.eye[2]};
+        pitch = 2.0f * c.tan_half_fovy / (float)c.height *
+                fabsf(q[0] * c.fwd[0] + q[1] * c.fwd[1] + q[2] * c.fwd[2]);
+    }
+    if (pitch <= 0.2f) return false;
+    const TileRays r = tile_rays(c, x0, y0);
+    auto fits = [&](auto mc, int na, int nb, int nm) {
+        constexpr int M = decltype(mc)::value, A = M == 0 ? 1 : 0, B = M == 2 ? 1 : 2;
+        TileLines<M> L;
+        if (!tile_lines<M>(r, L)) return false;
+        const float m = 0.5f * (float)(nm - 1);
+        float ext[2];
+        for (int k = 0; k < 2; ++k) {
+            const int ax = k == 0 ? A : B;
+            float lo = INFINITY, hi = -INFINITY;
+            for (int i = 0; i < 4; ++i)
+                for (int j = 0; j < 2; ++j) {
+                    const float p = L.B[i][ax] * (m + (float)j) + L.A[i][ax];
+                    lo = fminf(lo, p);
+                    hi = fmaxf(hi, p);
+                }
+            ext[k] = fminf(hi - lo + 2.0f, (float)(k == 0 ? na : nb));
+        }
+        if (M == 0) return ceilf(ext[0] / kSlabRows) * kSlabRows * ext[1] * G::kBXx <= 0.75f * G::kStageElems;
+        const bool hbm = (double)nx * ny * nz * G::kBytes > 128e6;
+        return ext[0] <= (hbm ? 50.0f : (float)(G::kBXw - 2)) &&
+               2.0f * ext[1] * (float)(ext[0] + 3.0f <= G::kBXn ? G::kBXn : G::kBXw) <= (float)G::kStageElems;
+    };
+    if (r.major == 0) return fits(std::integral_constant<int, 0>{}, ny, nz, nx);
+    if (r.major == 1) return fits(std::integral_constant<int, 1>{}, nx, nz, ny);
+    return fits(std::integral_constant<int, 2>{}, nx, ny, nz);
 }
 
 // The launch for one storage: the tensor maps (x-major chunks; y- and z-major chunks, narrow
