@@ -62,111 +62,152 @@ __device__ __forceinline__ void scatter_trilinear(float *gv, int nx, int ny, int
     }
 }
 
+// Shared memory of a CTA: the colour map, and one set of colour-map sums per warp: entry i's
+// sums of (1 - f) dL/dc (its own share of the samples between knots i and i + 1) and of f dL/dc
+// (its upper neighbour's share), 8 floats together.
+constexpr int kBwdWarps = kBwdThreads / 32, kBwdSums = kLut * 8;
+constexpr size_t kBwdSmem = sizeof(float4) * kLut + sizeof(float) * kBwdWarps * kBwdSums;
+
+// One CTA per 16 x 16 pixels, one ray per thread.
+//
+// What bounds it: the scatter.  A sample adds to 8 voxels (global reductions that nothing waits
+// for) and to 8 colour-map sums; as shared-memory float atomics, which are compare-and-swap
+// loops on addresses that the rays of a CTA share, the latter took most of the time (256^3 cube,
+// 512 x 512: 3.52 ms, 86 % of the shared-memory pipe, half the instructions).  Here every warp
+// has its own sums and its lanes add to them in turns: __match_any_sync groups the lanes by
+// entry, each lane's rank in its group is its turn, and the turns (the largest group: 3 to 4)
+// are plain 16-byte loads, adds and stores.  Lanes of a warp therefore step together.
 template <int INTERP>
 __global__ void __launch_bounds__(kBwdThreads) backward_kernel(SamplerF32<long long> s, shw_camera cam,
                                                                    BackwardArgs a)
 {
-    __shared__ float4 lut_s[kLut];
-    __shared__ float glut_s[kLut * 4];
+    extern __shared__ __align__(16) unsigned char bwd_smem[];
+    float4 *lut_s = reinterpret_cast<float4 *>(bwd_smem);
+    float *sums = reinterpret_cast<float *>(bwd_smem + sizeof(float4) * kLut);
     __shared__ float gs_s;
     for (int i = threadIdx.x; i < kLut; i += blockDim.x) lut_s[i] = a.lut[i];
-    for (int i = threadIdx.x; i < kLut * 4; i += blockDim.x) glut_s[i] = 0.0f;
+    for (int i = threadIdx.x; i < kBwdWarps * kBwdSums; i += blockDim.x) sums[i] = 0.0f;
     if (threadIdx.x == 0) gs_s = 0.0f;
     __syncthreads();
+    float4 *mine = reinterpret_cast<float4 *>(sums + (threadIdx.x >> 5) * kBwdSums);
+    const int lane = threadIdx.x & 31;
 
     float gs = 0.0f;
     int px, py;
     bwd_pixel(px, py);
-    if (px < a.width && py < a.height) {
-        const long long pix = (long long)py * a.width + px;
-        const long long npix = (long long)a.width * a.height;
-        RayFx r;
-        const bool hit = setup_ray(cam, px, py, s.nx, s.ny, s.nz, a.step, r);
-        const int K = hit ? min(min(a.ckpt_K[pix], r.N), a.nmax) : 0;
-        const float4 g = a.grad_rgba[pix];
-        float gT = -g.w;  // alpha_out = 1 - T_K
-        const int I = a.ckpt_interval;
-        float vseg[kMaxCkptInterval], Tseg[kMaxCkptInterval];
-        for (int m = (K - 1) / I; K > 0 && m >= 0; --m) {
-            const int k0 = m * I, k1 = min(k0 + I, K);
-            // recompute the segment forward from its checkpoint
-            float T = (m < a.nckpt) ? a.ckpt_T[(long long)m * npix + pix] : 0.0f;
-            for (int j = 0; j < k1 - k0; ++j) {
-                const long long X = r.P[0] + (long long)(k0 + j) * r.D[0];
-                const long long Y = r.P[1] + (long long)(k0 + j) * r.D[1];
-                const long long Z = r.P[2] + (long long)(k0 + j) * r.D[2];
-                const float v = fetch<INTERP>(s, X, Y, Z);
-                vseg[j] = v;
-                Tseg[j] = T;
-                const float vv = isnan(v) ? a.lo : v;
-                const float4 c = lut_eval(lut_s, normalise(vv, a.lo, a.inv_range));
-                const float al = __saturatef(a.opacity_scale * c.w);
-                T = T * (1.0f - al);
-            }
-            // walk it backwards
-            for (int j = k1 - k0 - 1; j >= 0; --j) {
-                const float v = vseg[j];
-                const bool nan = isnan(v);
-                const float vv = nan ? a.lo : v;
-                const float x = (vv - a.lo) * a.inv_range;
-                const float vh = __saturatef(x);
-                const float u = vh * 255.0f;
-                const int i0 = min(__float2int_rd(u), 254);
-                const float f = u - (float)i0;
-                const float4 L0 = lut_s[i0], L1 = lut_s[i0 + 1];
-                const float4 c = make_float4(lerp(L0.x, L1.x, f), lerp(L0.y, L1.y, f), lerp(L0.z, L1.z, f),
-                                             lerp(L0.w, L1.w, f));
-                const float alpha = a.opacity_scale * c.w;
-                const float al = __saturatef(alpha);
-                const float Tk = Tseg[j];
-                const float ga = (g.x * c.x + g.y * c.y + g.z * c.z) * Tk - gT * Tk;
-                const float wc = Tk * al;
-                const float gcr = g.x * wc, gcg = g.y * wc, gcb = g.z * wc;
-                gT = gT * (1.0f - al) + al * (g.x * c.x + g.y * c.y + g.z * c.z);
-                const float galpha = (alpha >= 0.0f && alpha <= 1.0f) ? ga : 0.0f;
-                gs = __fmaf_rn(galpha, c.w, gs);
-                const float gca = galpha * a.opacity_scale;
-                if (a.grad_lut != nullptr) {
-                    const float w0 = 1.0f - f;
-                    float *q0 = glut_s + 4 * i0, *q1 = glut_s + 4 * (i0 + 1);
-                    atomicAdd(q0 + 0, w0 * gcr);
-                    atomicAdd(q0 + 1, w0 * gcg);
-                    atomicAdd(q0 + 2, w0 * gcb);
-                    atomicAdd(q0 + 3, w0 * gca);
-                    atomicAdd(q1 + 0, f * gcr);
-                    atomicAdd(q1 + 1, f * gcg);
-                    atomicAdd(q1 + 2, f * gcb);
-                    atomicAdd(q1 + 3, f * gca);
+    const bool inside = px < a.width && py < a.height;
+    const long long pix = inside ? (long long)py * a.width + px : 0;
+    const long long npix = (long long)a.width * a.height;
+    RayFx r;
+    const bool hit = inside && setup_ray(cam, px, py, s.nx, s.ny, s.nz, a.step, r);
+    const int K = hit ? min(min(a.ckpt_K[pix], r.N), a.nmax) : 0;
+    const float4 g = hit ? a.grad_rgba[pix] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    float gT = -g.w;  // alpha_out = 1 - T_K
+    const int I = a.ckpt_interval;
+    float vseg[kMaxCkptInterval], Tseg[kMaxCkptInterval];
+    const int Kw = (int)__reduce_max_sync(0xffffffffu, (unsigned)K);  // the warp's longest ray
+    for (int m = Kw > 0 ? (Kw - 1) / I : -1; m >= 0; --m) {
+        const int k0 = m * I, n = min(max(K - k0, 0), I), nw = min(Kw - k0, I);
+        // recompute the segment forward from its checkpoint
+        float T = (n > 0 && m < a.nckpt) ? a.ckpt_T[(long long)m * npix + pix] : 0.0f;
+        for (int j = 0; j < n; ++j) {
+            const long long X = r.P[0] + (long long)(k0 + j) * r.D[0];
+            const long long Y = r.P[1] + (long long)(k0 + j) * r.D[1];
+            const long long Z = r.P[2] + (long long)(k0 + j) * r.D[2];
+            const float v = fetch<INTERP>(s, X, Y, Z);
+            vseg[j] = v;
+            Tseg[j] = T;
+            const float vv = isnan(v) ? a.lo : v;
+            const float4 c = lut_eval(lut_s, normalise(vv, a.lo, a.inv_range));
+            const float al = __saturatef(a.opacity_scale * c.w);
+            T = T * (1.0f - al);
+        }
+        __syncwarp();
+        // walk it backwards, the warp's lanes together (a shorter ray joins at its own end)
+        for (int j = nw - 1; j >= 0; --j) {
+            const bool on = j < n;
+            const float v = on ? vseg[j] : a.lo;
+            const bool nan = isnan(v);
+            const float vv = nan ? a.lo : v;
+            const float x = (vv - a.lo) * a.inv_range;
+            const float vh = __saturatef(x);
+            const float u = vh * 255.0f;
+            const int i0 = min(__float2int_rd(u), 254);
+            const float f = u - (float)i0;
+            const float4 L0 = lut_s[i0], L1 = lut_s[i0 + 1];
+            const float4 c = make_float4(lerp(L0.x, L1.x, f), lerp(L0.y, L1.y, f), lerp(L0.z, L1.z, f),
+                                         lerp(L0.w, L1.w, f));
+            const float alpha = a.opacity_scale * c.w;
+            const float al = __saturatef(alpha);
+            const float Tk = on ? Tseg[j] : 0.0f;
+            const float gc = g.x * c.x + g.y * c.y + g.z * c.z;
+            const float ga = gc * Tk - gT * Tk;
+            const float wc = Tk * al;
+            const float gcr = g.x * wc, gcg = g.y * wc, gcb = g.z * wc;
+            if (on) gT = gT * (1.0f - al) + al * gc;
+            const float galpha = (on && alpha >= 0.0f && alpha <= 1.0f) ? ga : 0.0f;
+            gs = __fmaf_rn(galpha, c.w, gs);
+            const float gca = galpha * a.opacity_scale;
+            if (a.grad_lut != nullptr) {
+                // lanes on the same entry take turns (a lane without a sample has an entry of its own)
+                const unsigned same = __match_any_sync(0xffffffffu, on ? i0 : kLut + lane);
+                const int turn = on ? __popc(same & ((1u << lane) - 1u)) : 0;
+                const int turns = __reduce_max_sync(0xffffffffu, turn);
+                const float w0 = 1.0f - f;
+                for (int t = 0; t <= turns; ++t) {
+                    if (on && turn == t) {
+                        float4 q0 = mine[2 * i0], q1 = mine[2 * i0 + 1];
+                        q0.x += w0 * gcr;
+                        q0.y += w0 * gcg;
+                        q0.z += w0 * gcb;
+                        q0.w += w0 * gca;
+                        q1.x += f * gcr;
+                        q1.y += f * gcg;
+                        q1.z += f * gcb;
+                        q1.w += f * gca;
+                        mine[2 * i0] = q0;
+                        mine[2 * i0 + 1] = q1;
+                    }
+                    __syncwarp();
                 }
-                if (a.grad_vol != nullptr && !nan) {
-                    const float gvh = 255.0f * (gcr * (L1.x - L0.x) + gcg * (L1.y - L0.y) + gcb * (L1.z - L0.z) +
-                                                gca * (L1.w - L0.w));
-                    const float gv = (x >= 0.0f && x <= 1.0f) ? gvh * a.inv_range : 0.0f;
-                    if (gv != 0.0f) {
-                        const long long X = r.P[0] + (long long)(k0 + j) * r.D[0];
-                        const long long Y = r.P[1] + (long long)(k0 + j) * r.D[1];
-                        const long long Z = r.P[2] + (long long)(k0 + j) * r.D[2];
-                        if constexpr (INTERP == SHW_NEAREST) {
-                            const int xi = clampi(fx_round(X), 0, s.nx - 1), yi = clampi(fx_round(Y), 0, s.ny - 1),
-                                      zi = clampi(fx_round(Z), 0, s.nz - 1);
-                            atomicAdd(a.grad_vol + ((size_t)zi * s.nx * s.ny + (size_t)yi * s.nx + xi), gv);
-                        } else {
-                            scatter_trilinear(a.grad_vol, s.nx, s.ny, s.nz, X, Y, Z, gv);
-                        }
+            }
+            if (a.grad_vol != nullptr && on && !nan) {
+                const float gvh = 255.0f * (gcr * (L1.x - L0.x) + gcg * (L1.y - L0.y) + gcb * (L1.z - L0.z) +
+                                            gca * (L1.w - L0.w));
+                const float gv = (x >= 0.0f && x <= 1.0f) ? gvh * a.inv_range : 0.0f;
+                if (gv != 0.0f) {
+                    const long long X = r.P[0] + (long long)(k0 + j) * r.D[0];
+                    const long long Y = r.P[1] + (long long)(k0 + j) * r.D[1];
+                    const long long Z = r.P[2] + (long long)(k0 + j) * r.D[2];
+                    if constexpr (INTERP == SHW_NEAREST) {
+                        const int xi = clampi(fx_round(X), 0, s.nx - 1), yi = clampi(fx_round(Y), 0, s.ny - 1),
+                                  zi = clampi(fx_round(Z), 0, s.nz - 1);
+                        atomicAdd(a.grad_vol + ((size_t)zi * s.nx * s.ny + (size_t)yi * s.nx + xi), gv);
+                    } else {
+                        scatter_trilinear(a.grad_vol, s.nx, s.ny, s.nz, X, Y, Z, gv);
                     }
                 }
             }
         }
     }
-    // block reduction of the colour-map and scale gradients: warp shuffles, then one
-    // shared atomic per warp, then one global atomic per entry per CTA
+    // the scale gradient: warp shuffles, then one shared atomic per warp; the colour map's: the
+    // warps' sums of an entry's own share and its lower neighbour's upper share; one global atomic
+    // per entry per CTA
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) gs += __shfl_xor_sync(0xffffffffu, gs, o);
-    if ((threadIdx.x & 31) == 0) atomicAdd(&gs_s, gs);
+    if (lane == 0) atomicAdd(&gs_s, gs);
     __syncthreads();
     if (a.grad_lut != nullptr)
-        for (int i = threadIdx.x; i < kLut * 4; i += blockDim.x)
-            if (glut_s[i] != 0.0f) atomicAdd(a.grad_lut + i, glut_s[i]);
+        for (int i = threadIdx.x; i < kLut * 4; i += blockDim.x) {
+            const int e = i >> 2, ch = i & 3;
+            float v = 0.0f;
+            for (int w = 0; w < kBwdWarps; ++w) {
+                const float *q = sums + w * kBwdSums + 8 * e + ch;
+                v += q[0];
+                if (e > 0) v += q[-4];
+            }
+            if (v != 0.0f) atomicAdd(a.grad_lut + i, v);
+        }
     if (threadIdx.x == 0 && a.grad_scale != nullptr) atomicAdd(a.grad_scale, gs_s);
 }
 
@@ -220,9 +261,11 @@ extern "C" shw_status shw_render_backward(const shw_volume *vol, const shw_camer
                             (long long)vol->nx * vol->ny};
     const dim3 grid((unsigned)ceil_div(cam->width, kBwdTile), (unsigned)ceil_div(cam->height, kBwdTile));
     cudaStream_t st = as_stream(stream);
-    if (p->interp == SHW_NEAREST)
-        backward_kernel<SHW_NEAREST><<<grid, kBwdThreads, 0, st>>>(s, *cam, a);
-    else
-        backward_kernel<SHW_TRILINEAR><<<grid, kBwdThreads, 0, st>>>(s, *cam, a);
+    auto kern = p->interp == SHW_NEAREST ? backward_kernel<SHW_NEAREST> : backward_kernel<SHW_TRILINEAR>;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBwdSmem) != cudaSuccess) {
+        cudaGetLastError();
+        return SHW_ECUDA;
+    }
+    kern<<<grid, kBwdThreads, kBwdSmem, st>>>(s, *cam, a);
     return after_launch();
 }
