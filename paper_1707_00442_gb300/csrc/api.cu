@@ -397,13 +397,12 @@ shw_status shw_render(const shw_volume *vol, const shw_volume *vol2, const shw_c
         if (ss != SHW_EUNSUPPORTED || debug(SHW_DEBUG_REQUIRE_STAGING)) return ss;
         return render_pair(p->mode, p->interp, *vol, *cam, a, st);
     }
-    // in-ray smoothing of one float32 cube: the rolling marcher, when it applies (512^3 on
-    // 1000 x 1000, MIP: 9 taps per axis 53.9 -> 11.5 ms, the 5-box 5.86 -> 2.32 ms)
+    // in-ray smoothing of one float32 cube: the rolling marcher, when it applies and pays
     if (p->smooth != SHW_SMOOTH_NONE && sto == SHW_F32 && v2 == nullptr) {
-        const shw_status ss = a.box_lattice == 2       ? render_roll_box(p->mode, p->interp, *vol, *cam, a, st)
+        const shw_status ss = a.box_lattice == 2             ? render_roll_box(p->mode, p->interp, *vol, *cam, a, st)
                               : p->smooth == SHW_SMOOTH_TAPS ? render_roll_taps(p->mode, p->interp, *vol, *cam, a, st)
                                                              : SHW_EUNSUPPORTED;
-        if (ss != SHW_EUNSUPPORTED) return ss;
+        if (ss != SHW_EUNSUPPORTED || debug(SHW_DEBUG_REQUIRE_STAGING)) return ss;
     }
     if (a.box_lattice == 2)
         return vol->storage == SHW_F32 ? render_smooth_lat_f32(p->mode, p->interp, *vol, *cam, a, st)

@@ -988,13 +988,13 @@ shw_status launch_render_modes(int mode, int interp, const S &s, const S &s2, co
     const int nsm = sm_count();
     const int nwarp_tiles = (int)(tiles * kCtaWarps);
     // persistent grid: as many CTAs as fit on the device at once (at most one per tile).  An
-    // image of only a few tiles per CTA takes fewer CTAs, down to 8 per SM: more would leave
+    // image of only a few tiles per CTA takes fewer of the raised counts, down to 8 per SM: more would leave
     // nothing to even out the long rays with (128^3 on 500 x 500, compositing: 137 us with 8 per
     // SM, 193 with 12; 1000 x 1000: 389 and 383).  Nearest sampling's rays are too short to
     // mind (45 us with 11 per SM, 53 with 8).
-    auto persistent = [&](auto kern, int per_sm) {
+    auto persistent = [&](auto kern, int per_sm, bool more_ctas) {
         long long g = std::min<long long>((long long)per_sm * nsm, tiles);
-        if (SMK == 0 && interp != SHW_NEAREST) g = std::min(g, std::max(tiles / 4, 8LL * nsm));
+        if (SMK == 0 && interp != SHW_NEAREST && more_ctas) g = std::min(g, std::max(tiles / 4, 8LL * nsm));
         kern<<<(unsigned)std::max<long long>(g, 1), block, 0, st>>>(s, s2, cam, a, ctr, nwarp_tiles);
     };
     if (SMK > 0 && (ctr == nullptr || nsm <= 0)) return SHW_ECUDA;
@@ -1002,10 +1002,10 @@ shw_status launch_render_modes(int mode, int interp, const S &s, const S &s2, co
     do {                                                                       \
         if constexpr (SMK > 0)                                                 \
             persistent(render_kernel_persistent<M, I, S, SMK>,                 \
-                       resident_per_sm<render_kernel_persistent<M, I, S, SMK>>()); \
+                       resident_per_sm<render_kernel_persistent<M, I, S, SMK>>(), false); \
         else if (ctr != nullptr && nsm > 0)                                    \
             persistent(render_kernel_persistent<M, I, S>,                      \
-                       resident_per_sm<render_kernel_persistent<M, I, S>>());  \
+                       resident_per_sm<render_kernel_persistent<M, I, S>>(), render_min_ctas<M, I, 0>() > 8); \
         else                                                                   \
             render_kernel<M, I, S><<<grid, block, 0, st>>>(s, s2, cam, a);     \
     } while (0)

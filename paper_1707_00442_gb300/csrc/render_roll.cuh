@@ -93,6 +93,7 @@ struct RollShared {
     // cell c of a step: the lateral cells [x, x + y) along A and [z, z + w) along B whose
     // corners and taps the planes of its window all hold
     int4 range[kRollTable];
+    int dead[kDeadSlots];  // (SlabShared)
     int quit;
     int pad[3];
 };
@@ -188,7 +189,7 @@ struct RollRing {
                 return false;
         return true;
     }
-    __device__ __forceinline__ bool post_plain(int type, int tile)
+    __device__ __forceinline__ bool post_plain(int type, int tile, int seq = 0)
     {
         if (!drain_to(posts - kRollBars)) return false;
         const int st = posts % kRollBars;
@@ -196,6 +197,8 @@ struct RollRing {
             RollHdr h{};
             h.type = type;
             h.tile = tile;
+            h.m0 = seq;
+            if (type == kStageTile) sh.dead[seq % kDeadSlots] = 0;
             sh.hdr[st] = h;
             mbar_arrive(&sh.full[st]);
         }
@@ -282,7 +285,7 @@ __device__ __forceinline__ void roll_xplanes(const RollArgs &ra, const RollGeom 
 
 template <int M>
 __device__ __forceinline__ bool roll_produce(const TileRays &r, bool persp, const CUtensorMap *map,
-                                             const RenderArgs &a, const RollArgs &ra, int tile, float *stage,
+                                             const RenderArgs &a, const RollArgs &ra, int tile, int seq, float *stage,
                                              RollRing &ring)
 {
     using AX = RollAxes<M>;
@@ -320,7 +323,8 @@ __device__ __forceinline__ bool roll_produce(const TileRays &r, bool persp, cons
     const int before = ring.posts - 2;  // the last post before this tile's start: it may read the ring
     bool fresh = true;
     int have_lo = 0, have_hi = -1;  // slots staged
-    for (int m0 = floor_div(dir > 0 ? first : last, s) * s; dir > 0 ? m0 <= last : m0 + s > first; m0 += dir * s) {
+    for (int m0 = floor_div(dir > 0 ? first : last, s) * s; (dir > 0 ? m0 <= last : m0 + s > first) && !tile_dead(sh.dead, seq);
+         m0 += dir * s) {
         const int plo = max(m0 - H, 0), phi = min(m0 + s + H, n_m - 1);
         const int slo = plo / g, shi = phi / g;
         const int c0 = fresh ? slo : (dir > 0 ? have_hi + 1 : slo), c1 = fresh ? shi : (dir > 0 ? shi : have_lo - 1);
@@ -421,7 +425,7 @@ __device__ __forceinline__ void roll_producer(const CUtensorMap *maps, const shw
     RollRing ring{sh, ra};
     const int on[3] = {ra.geo[0].on, ra.geo[1].on, ra.geo[2].on};
     bool ok = true;
-    while (ok) {
+    for (int seq = 0; ok; ++seq) {
         unsigned t = 0;
         if (lane == 0) t = atomicAdd(ra.ctr, 1u);
         t = __shfl_sync(0xffffffffu, t, 0);
@@ -429,17 +433,17 @@ __device__ __forceinline__ void roll_producer(const CUtensorMap *maps, const shw
             ring.post_plain(kStageExit, 0);
             break;
         }
-        if (!ring.post_plain(kStageTile, (int)t)) break;
+        if (!ring.post_plain(kStageTile, (int)t, seq)) break;
         int tx, ty;
         slab_tile((int)t, a, tx, ty);
         const TileRays r = roll_rays(cam, tx * kSlabTW, ty * kSlabTH, on, ra.xbias);
         const bool persp = !cam.ortho;
         if (r.major == 0)
-            ok = roll_produce<0>(r, persp, nullptr, a, ra, (int)t, stage, ring);
+            ok = roll_produce<0>(r, persp, nullptr, a, ra, (int)t, seq, stage, ring);
         else if (r.major == 1)
-            ok = roll_produce<1>(r, persp, &maps[0], a, ra, (int)t, stage, ring);
+            ok = roll_produce<1>(r, persp, &maps[0], a, ra, (int)t, seq, stage, ring);
         else
-            ok = roll_produce<2>(r, persp, &maps[1], a, ra, (int)t, stage, ring);
+            ok = roll_produce<2>(r, persp, &maps[1], a, ra, (int)t, seq, stage, ring);
         if (ok) ok = ring.post_plain(kStageTileEnd, (int)t);
     }
     // no exit while a copy into this CTA's shared memory is in flight: wait (bounded) for the
@@ -662,7 +666,8 @@ __device__ __forceinline__ void roll_consumer(const S &s, const shw_camera &cam,
     RayFx r;
     long long pix = 0;
     int N = 0;
-    bool has = false, live = false;
+    bool has = false, live = false, said = false;
+    int seq = 0;
     for (int posts = 0;; ++posts) {
         const int si = posts % kRollBars;
         if (!slab_wait(&sh.full[si], (uint32_t)((posts / kRollBars) & 1), quit, ra.err, ra.polls)) return;
@@ -677,6 +682,8 @@ __device__ __forceinline__ void roll_consumer(const S &s, const shw_camera &cam,
             const bool hit = has && !quick_miss(cam, px, py, s.nx, s.ny, s.nz) &&
                              setup_ray(cam, px, py, s.nx, s.ny, s.nz, a.step, r);
             N = hit ? min(r.N, a.nmax) : 0;
+            seq = h.m0;
+            said = false;
             live = N > 0;
             q.st = typename RollMarch<MODE, KIND>::St{};
             q.done = 0;
@@ -727,6 +734,7 @@ __device__ __forceinline__ void roll_consumer(const S &s, const shw_camera &cam,
             has = false;
         }
         __syncwarp();
+        if (h.type != kStageTileEnd) report_dead(sh.dead, seq, live && q.k < q.kend, said);
         if (lane == 0) mbar_arrive(&sh.empty[si]);
     }
 }
@@ -888,6 +896,22 @@ shw_status roll_launch_one(const RollMaps &maps, const S &s, const shw_camera &c
     return after_launch();
 }
 
+// Whether the ring pays (else the samples are gathered): its hand-overs and halo planes are a
+// fixed cost per tile, and the gathers of a small cube hit the caches.  Over 864 renders (32^3 ..
+// 320^3 and oblong cubes, 128^2 .. 1000 x 800, three views) the rule is 2 to 4 % from the better of
+// the two marchers; for 9 taps always gathering is 24 % off and never 12 %, for the box 5 % and
+// 42 %.  Below 64 voxels on an axis most samples' taps clamp; few taps (1 pair) and row copies
+// need a larger cube, and the box, two fetches a sample when gathered, needs 10^7 voxels and
+// tensor copies (512^3 on 1000 x 1000: 9 taps 53.9 ms gathered, 11.5 staged; the 5-box 5.86 and
+// 2.32).
+template <int KIND>
+inline bool roll_pays(const int n[3], bool tmaps, int ntaps)
+{
+    const double vox = (double)n[0] * n[1] * n[2];
+    if (KIND == kRollBox) return tmaps && vox >= 1e7;
+    return std::min(n[0], std::min(n[1], n[2])) >= 64 && ((tmaps && ntaps >= 2) || vox >= 2e6);
+}
+
 // In-ray smoothing of a float32 cube through the rolling marcher; SHW_EUNSUPPORTED when it
 // does not serve the request.
 template <int KIND>
@@ -905,6 +929,7 @@ shw_status roll_launch(int mode, const shw_volume &v, const shw_camera &cam, con
             ra.halo = std::max(ra.halo, (int)((o + 0xffffffffLL) >> 32));
         }
     const bool tmaps = v.nx % 4 == 0 && aligned(v.data, 16);
+    if (!debug(SHW_DEBUG_REQUIRE_STAGING) && !roll_pays<KIND>(n, tmaps, a0.smooth_n)) return SHW_EUNSUPPORTED;
     ra.rows = !tmaps;
     ra.goff = (int)((reinterpret_cast<uintptr_t>(v.data) >> 2) & 3);
     size_t extra = sizeof(RollShared);

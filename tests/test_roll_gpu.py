@@ -1,7 +1,8 @@
 """The rolling marcher (in-ray smoothing from a ring of cube planes in shared memory) on the GPU.
 
 It fetches the gather marcher's corners at the same fixed-point positions and sums the taps in
-the same order, so every output must equal the gather marcher's bit for bit: views whose major
+the same order, so every output must equal the gather marcher's bit for bit (it is forced with
+SHW_DEBUG_REQUIRE_STAGING, also where gathering would be faster): views whose major
 axis is x, y or z, both directions, parallel and perspective, the eye inside the cube; rows
 that are and are not 16-byte multiples, a cube that starts off a 16-byte boundary (bulk copies
 of rows); reaches from none to more than the ring holds; cubes smaller than the reach."""
@@ -54,10 +55,14 @@ def _cube(dims, offset):
 def _same(m, vol, cam, mode, what, **kw):
     lut = to_dev(scene.linear_lut())
     outs = []
-    for flags in ((), ("no_staging",)):
-        with m.debug_flags(*flags):
+    for flags in (("require_staging",), ("no_staging",)):
+        try:
+            with m.debug_flags(*flags):
+                outs.append(m.render(vol, cam, mode, lut=lut, **kw))
+                torch.cuda.synchronize()
+        except m.ShwError as e:  # a footprint that no ring holds: the default route serves it
+            assert e.status == 2 and flags == ("require_staging",)
             outs.append(m.render(vol, cam, mode, lut=lut, **kw))
-            torch.cuda.synchronize()
         m.sync_status()
     for k in outs[0]:
         a, b = outs[0][k].cpu().numpy(), outs[1][k].cpu().numpy()
