@@ -15,7 +15,7 @@ static bool axis_eligible(const shw_volume &v, const shw_camera &c, int mode)
 {
     if (debug(SHW_DEBUG_NO_AXIS_SWEEP)) return false;
     return v.storage == SHW_F32 && mode != SHW_RATIO && mode <= SHW_MOMENT1 && c.ortho && c.fwd[0] == 0.0f && c.fwd[1] == 0.0f &&
-           c.fwd[2] != 0.0f && c.right[2] == 0.0f && c.up[2] == 0.0f && v.nx % 4 == 0 && aligned(v.data, 16) &&
+           c.fwd[2] != 0.0f && c.right[2] == 0.0f && c.up[2] == 0.0f &&
            (long long)v.nx * v.ny < (1ll << 29);  // byte offsets in a plane fit an int
 }
 
@@ -40,13 +40,20 @@ shw_status render_axis(int mode, int interp, const shw_volume &v, const shw_came
     // corner and the interpolation neighbour, and up to 3 to align the x start to 16 bytes
     A.bw = ((int)std::ceil(ext_x) + 8 + 3) & ~3;
     A.bh = (int)std::ceil(ext_y) + 6;
-    const bool fix = A.bw <= kFixBW && A.bh <= kFixBH;
+    // rows that no tensor copy takes: row copies, with 32-bit element indexes
+    A.rows = v.nx % 4 != 0 || !aligned(v.data, 16);
+    if (A.rows && (long long)v.nx * v.ny * v.nz >= (1ll << 31)) return SHW_EUNSUPPORTED;
+    const bool fix = A.bw <= kFixBW && A.bh <= kFixBH && !A.rows;
     if (fix) {
         A.bw = kFixBW;
         A.bh = kFixBH;
     }
     if (A.bw > 256 || A.bh > 256) return SHW_EUNSUPPORTED;  // the tensor copy's box limit
-    A.stage_stride = fix ? kFixStride : (A.bw * A.bh + 31) & ~31;  // TMA destinations start on 128 bytes
+    // (a row copy brings whole 16-byte pieces, up to 10 floats more than the box)
+    A.pitch = A.rows ? A.bw + 10 + ((v.nx - A.bw - 10) & 3) : A.bw;
+    A.goff = (int)((reinterpret_cast<uintptr_t>(v.data) >> 2) & 3);
+    // TMA destinations start on 128 bytes
+    A.stage_stride = fix ? kFixStride : (A.pitch * A.bh + (A.rows ? 16 : 0) + 31) & ~31;
     const int kmode = (mode == SHW_MIP && a.index == nullptr) ? kMipValue : mode;
     const size_t smem = (size_t)axis_stages(kmode, fix) * A.stage_stride * 4;
     if (smem > (size_t)kAxSmemLimit) return SHW_EUNSUPPORTED;
@@ -63,8 +70,8 @@ shw_status render_axis(int mode, int interp, const shw_volume &v, const shw_came
     A.tiles_x = ceil_div(c.width, kAxTX);
     const long long tiles = (long long)A.tiles_x * ceil_div(c.height, kAxTY);
     const float *data = static_cast<const float *>(v.data);
-    CUtensorMap map;
-    if (!encode_tmap_3d_f32(&map, data, v.nx, v.ny, v.nz, A.bw, A.bh)) return SHW_EUNSUPPORTED;
+    CUtensorMap map{};
+    if (!A.rows && !encode_tmap_3d_f32(&map, data, v.nx, v.ny, v.nz, A.bw, A.bh)) return SHW_EUNSUPPORTED;
     const bool up = c.fwd[2] > 0.0f;  // rays advance towards +z (the sign of every ray's z step)
     return fix ? launch_axis<true>(kmode, interp, up, map, data, c, a, A, (unsigned)tiles, smem, st)
                : launch_axis<false>(kmode, interp, up, map, data, c, a, A, (unsigned)tiles, smem, st);

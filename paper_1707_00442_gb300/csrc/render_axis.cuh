@@ -88,6 +88,9 @@ struct AxisArgs {
     float cx, ax, bx;  // pixel (px, py) -> x = cx + ax px + bx py (FP32, for the box only)
     float cy, ay, by;
     unsigned *err;
+    int rows;          // 1: planes by row copies (a cube whose rows no tensor copy takes; runtime boxes only)
+    int pitch;         // floats between box rows: bw, or with row copies congruent to nx modulo 4
+    int goff;          // row copies: floats from the 16-byte boundary below the cube to the cube
 };
 
 __device__ __forceinline__ float bilerp(float v00, float v01, float v10, float v11, float fx, float fy)
@@ -160,6 +163,96 @@ __device__ __forceinline__ void axis_emit(const RenderArgs &a, long long pix, bo
     if (a.nsamples) a.nsamples[pix] = done;
 }
 
+// Row copies: stage index of the box's first element for plane pz (4 to 7), congruent to its
+// global index modulo 4, so that 16-byte pieces stay 16-byte pieces.
+__device__ __forceinline__ int axis_pad(const AxisArgs &A, int x0, int y0, int pz)
+{
+    return 4 + ((A.goff + (pz * (A.ny & 3) + y0) * (A.nx & 3) + x0) & 3);
+}
+
+// The producer warp of a sweep by row copies: the tensor copies' ring, every lane bringing pieces
+// of the box's rows (a cube of 350 x 350 x 454, 350^2 pixels, MIP: 786 us by the gather marcher,
+// the only other one for such rows; 120 us by tensor copies for 348 x 348).
+template <int S, int G, bool UP>
+__device__ __forceinline__ void axis_rows(float *sm, uint64_t *full, uint64_t *empty, volatile int &quit,
+                                          const float *vol, const AxisArgs &A, int x0, int y0, int p_first, int nplanes)
+{
+    const int lane = threadIdx.x & 31;
+    const unsigned plane = (unsigned)A.nx * A.ny, nvox = plane * (unsigned)A.nz;
+    const int len = min(A.bw, A.nx - x0), nr = min(A.bh, A.ny - y0), np = (len + 6) / 4;  // pieces of a row, at most
+    const int total = nr * np;
+    // this lane's pieces: the first, and from one to the next (32 further)
+    const int row0 = lane / np, piece0 = lane - row0 * np, drow = 32 / np, dpiece = 32 - drow * np;
+    int issued = 0;
+    for (int j = 0; j < nplanes; j += G) {
+        const int s = j & (S - 1);
+        if (j >= S) {  // wait until every consumer warp has released the group j - S
+            const uint32_t par = (uint32_t)(((j / S) - 1) & 1);
+            bool ok = false, stop = false;
+            for (int it = 0; it < kAxWaitPolls && !ok && !stop; ++it) {
+                ok = __all_sync(0xffffffffu, mbar_try_wait_sleep(&empty[s], par, kAxSleepNs));
+                stop = !ok && __any_sync(0xffffffffu, quit != 0);
+            }
+            if (!ok) {
+                if (!stop && lane == 0) {
+                    atomicOr(A.err, kErrWaitTimeout);
+                    quit = 1;
+                }
+                break;
+            }
+        }
+        const int cnt = min(G, nplanes - j);
+        for (int e = 0; e < cnt; ++e) {
+            const int pz = UP ? p_first + j + e : p_first - j - e;
+            const unsigned g0 = (unsigned)pz * plane + (unsigned)(y0 * A.nx + x0), b = (unsigned)A.goff + g0;
+            float *stage = sm + (s + e) * A.stage_stride;
+            const int rz = (int)(b & 3u);  // the first element past a 16-byte boundary; stage index 4 + rz
+            int piece = piece0;
+            if (b >= (unsigned)A.goff + 3u && b + (unsigned)((nr - 1) * A.nx + len) + 8u <= (unsigned)A.goff + nvox) {
+                // whole pieces: row r's piece p starts at the boundary below element r nx + 4 p
+                // past the first, and in the stage likewise (pitches agree modulo 4)
+                const float *src = vol - A.goff + (b - (unsigned)rz);
+                int ga = rz + row0 * A.nx + 4 * piece0, sa = rz + row0 * A.pitch + 4 * piece0;
+                const int dg = drow * A.nx + 4 * dpiece, ds = drow * A.pitch + 4 * dpiece;
+                const int wg = A.nx - 4 * np, ws = A.pitch - 4 * np;
+#pragma unroll 4
+                for (int i = lane; i < total; i += 32) {
+                    cp_async16(stage + 4 + (sa & ~3), src + (ga & ~3));
+                    piece += dpiece;
+                    ga += dg;
+                    sa += ds;
+                    if (piece >= np) {
+                        piece -= np;
+                        ga += wg;
+                        sa += ws;
+                    }
+                }
+            } else {  // next to the ends of the cube's memory
+                int row = row0;
+                for (int i = lane; i < total; i += 32) {
+                    copy_piece(vol, (unsigned)A.goff, nvox, g0 + (unsigned)(row * A.nx), len, stage,
+                               4 + rz + row * A.pitch, piece);
+                    piece += dpiece;
+                    row += drow;
+                    if (piece >= np) {
+                        piece -= np;
+                        ++row;
+                    }
+                }
+            }
+        }
+        cp_async_arrive(&full[s]);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&full[s]);
+        issued = j + cnt;
+    }
+    // every copy issued lands before this CTA may exit (the groups still in the ring)
+    if (lane == 0)
+        for (int j = (max(issued - S, 0) + G - 1) & ~(G - 1); j < issued; j += G)
+            mbar_wait(&full[j & (S - 1)], (uint32_t)((j / S) & 1), A.err);
+    __syncwarp();
+}
+
 // MODE: a transfer function, or kMipValue.  UP: rays advance towards +z.  FIX: the
 // staged box is kFixBW x kFixBH (else A.bw x A.bh).  W: consumer warps.
 template <int MODE, int INTERP, bool UP, bool FIX, int W = axis_warps<MODE>()>
@@ -179,7 +272,8 @@ __global__ void __launch_bounds__(AxCfg<W>::threads, MODE == SHW_COMPOSITE ? 1 :
     const bool consumer = warp < W;
     const int tile = blockIdx.x, tyi = tile / A.tiles_x, txi = tile - tyi * A.tiles_x;
     const int bw = FIX ? kFixBW : A.bw, bh = FIX ? kFixBH : A.bh;
-    const int stride = FIX ? kFixStride : A.stage_stride;
+    const int stride = FIX ? kFixStride : A.stage_stride, pitch = FIX ? kFixBW : A.pitch;
+    const bool rows = !FIX && A.rows != 0;
 
     if (tid == 0) {
         s_any = 0;
@@ -196,10 +290,14 @@ __global__ void __launch_bounds__(AxCfg<W>::threads, MODE == SHW_COMPOSITE ? 1 :
         }
         s_x0 = ((int)floorf(xmin) - 2) & ~3;
         s_y0 = (int)floorf(ymin) - 2;
+        if (rows) {  // (row copies bring only rows and columns of the cube)
+            s_x0 = min(max((int)floorf(xmin) - 2, 0), A.nx - 1);
+            s_y0 = min(max(s_y0, 0), A.ny - 1);
+        }
         s_bad = 0;
         for (int s = 0; s < S; ++s) s_bad |= !tma_dst_ok(sm + s * stride, A.err);
         for (int s = 0; s < S; ++s) {
-            mbar_init(&full[s], 1);
+            mbar_init(&full[s], rows ? 33 : 1);  // (row copies: every producer lane's, and the post)
             mbar_init(&empty[s], W);
         }
         fence_barrier_init();
@@ -258,6 +356,10 @@ __global__ void __launch_bounds__(AxCfg<W>::threads, MODE == SHW_COMPOSITE ? 1 :
         // producer: one thread keeps the ring full, a group of G planes at a time -- planes
         // j .. j + G - 1 (j a multiple of G) go to stages s .. s + G - 1 and complete on stage
         // s's barrier, so each consumer warp waits and releases once per group
+        if (rows) {
+            axis_rows<S, G, UP>(sm, full, empty, s_quit, vol, A, x0b, y0b, p_first, nplanes);
+            return;
+        }
         if (lane != 0) return;
         const uint32_t plane_bytes = (uint32_t)(bw * bh * 4);
         int issued = 0;
@@ -318,10 +420,10 @@ __global__ void __launch_bounds__(AxCfg<W>::threads, MODE == SHW_COMPOSITE ? 1 :
             o00[i] = o01[i] = o10[i] = o11[i] = 0;
         } else if (c0 >= 0 && c1 < bw && r0 >= 0 && r1 < bh) {
             inbox |= 1 << i;
-            o00[i] = 4 * (r0 * bw + c0);
-            o01[i] = 4 * (r0 * bw + c1);
-            o10[i] = 4 * (r1 * bw + c0);
-            o11[i] = 4 * (r1 * bw + c1);
+            o00[i] = 4 * (r0 * pitch + c0);
+            o01[i] = 4 * (r0 * pitch + c1);
+            o10[i] = 4 * (r1 * pitch + c0);
+            o11[i] = 4 * (r1 * pitch + c1);
         } else {
             o00[i] = 4 * (gy0 * A.nx + gx0);
             o01[i] = 4 * (gy0 * A.nx + gx1);
@@ -332,7 +434,7 @@ __global__ void __launch_bounds__(AxCfg<W>::threads, MODE == SHW_COMPOSITE ? 1 :
     if constexpr (kChecked) {  // every offset inside the staged box, or inside the plane
 #pragma unroll
         for (int i = 0; i < R; ++i) {
-            const long long lim = ((inbox >> i) & 1) ? 4ll * bw * bh : 4ll * A.nx * A.ny;
+            const long long lim = ((inbox >> i) & 1) ? 4ll * pitch * bh : 4ll * A.nx * A.ny;
             const int lo = min(min(o00[i], o01[i]), min(o10[i], o11[i]));
             const int hi = max(max(o00[i], o01[i]), max(o10[i], o11[i]));
             const bool ok = lo >= 0 && (long long)hi + 4 <= lim;
@@ -361,6 +463,8 @@ __global__ void __launch_bounds__(AxCfg<W>::threads, MODE == SHW_COMPOSITE ? 1 :
     // which holds the sweep's plane jp
     auto load_plane = [&](int s, int jp, float2 pv[P]) {
         const char *t = reinterpret_cast<const char *>(sm + s * stride);
+        if constexpr (!FIX)
+            if (rows) t += 4 * axis_pad(A, x0b, y0b, UP ? p_first + jp : p_first - jp);
         if (all_inbox) {
 #pragma unroll
             for (int q = 0; q < P; ++q) {

@@ -63,6 +63,42 @@ __device__ __forceinline__ void tma_load_3d(void *dst, const CUtensorMap *map, i
         : "memory");
 }
 
+// 16 bytes (both addresses 16-byte aligned) or 4 into shared memory, asynchronously; the thread's
+// copies so far are then tied to `bar`, which counts one more arrival when they have landed
+// (cp_async_arrive: every thread of the barrier's count calls it, with copies or without).
+__device__ __forceinline__ void cp_async16(void *dst, const void *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async4(void *dst, const void *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_arrive(uint64_t *bar)
+{
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+
+// Piece j of a row copy: `len` floats from element `g` of a cube of nvox floats into
+// stage[at ...], in the 16-byte pieces that hold them (also the neighbours up to the next
+// 16-byte boundaries); at the two ends of the whole cube, where a piece would leave it, single
+// elements.  goff: floats from the 16-byte boundary below the cube to the cube; (goff + g) and
+// the stage index agree modulo 4 (stage 16-byte aligned).
+__device__ __forceinline__ void copy_piece(const float *cube, unsigned goff, unsigned nvox, unsigned g, int len,
+                                           float *stage, int at, int j)
+{
+    const unsigned g0 = goff + g, r = g0 & 3u, c = g0 - r + 4u * (unsigned)j;  // floats from the boundary
+    if (4 * j >= (int)r + len) return;
+    const float *src = cube - goff + c;
+    float *dst = stage + at - (int)r + 4 * j;
+    if (c >= goff && c + 4u <= goff + nvox) {
+        cp_async16(dst, src);
+    } else {
+        for (unsigned e = 0; e < 4u; ++e)
+            if (c + e >= goff && c + e < goff + nvox) cp_async4(dst + e, src + e);
+    }
+}
+
 // A tensor copy's shared-memory destination must start on 128 bytes: refuse (and
 // report) a copy that would not, instead of issuing it.
 __device__ __forceinline__ bool tma_dst_ok(const void *dst, unsigned *err)
