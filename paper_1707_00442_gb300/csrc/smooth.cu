@@ -209,9 +209,30 @@ constexpr int smooth_stage_floats()
     return ((kSmTY + 2 * R) * kSmBW + 31) & ~31;
 }
 
-template <int R, bool ZIP>
+// One plane of the staged box by 4-byte asynchronous copies (ROWS: a cube whose rows no tensor
+// copy takes), clamped to the edge on the way; 64 threads per row, the thread's own arrival on
+// `bar` once its copies have landed.  src: the plane.
+template <int R>
+__device__ __forceinline__ void copy_tile(float *tile, const float *src, int x0, int y0, int nx, int ny, int tid,
+                                          uint64_t *bar)
+{
+    const int c = tid & 63;
+    if (c < kSmBW) {
+        const float *col = src + clampi_s(x0 - kSmXP + c, 0, nx - 1);
+#pragma unroll
+        for (int row = tid >> 6; row < kSmTY + 2 * R; row += kSmThreads / 64)
+            cp_async4(tile + row * kSmBW + c, col + (size_t)clampi_s(y0 - R + row, 0, ny - 1) * nx);
+    }
+    cp_async_arrive(bar);
+}
+
+// ROWS: planes by copy_tile instead of a tensor copy, outputs by elements (a ragged row's
+// column pairs are not aligned).  401 x 300 x 300, r = 6: 247 us, 452 by the kernel without the
+// pipeline (400 x 300 x 300 by tensor copies: 200).
+template <int R, bool ZIP, bool ROWS>
 __global__ void __launch_bounds__(kSmThreads, smooth_min_blocks<R, ZIP>())
-    smooth_tma_kernel(const __grid_constant__ CUtensorMap tmap, float *__restrict__ out, int nx, int ny, int nz,
+    smooth_tma_kernel(const __grid_constant__ CUtensorMap tmap, const float *__restrict__ in, float *__restrict__ out,
+                      int nx, int ny, int nz,
                       int zchunk, SmoothWeights W, unsigned *err, const float *__restrict__ first, int skip_plane,
                       int polls)
 {
@@ -234,12 +255,16 @@ __global__ void __launch_bounds__(kSmThreads, smooth_min_blocks<R, ZIP>())
     if (tid == 0) {
         s_bad = 0;
         for (int s = 0; s < kSmStages; ++s) s_bad |= !tma_dst_ok(s_in + s * STAGE_FLOATS, err);
-        for (int s = 0; s < kSmStages; ++s) mbar_init(&bars[s], 1);
+        for (int s = 0; s < kSmStages; ++s) mbar_init(&bars[s], ROWS ? kSmThreads : 1);
         fence_barrier_init();
     }
     __syncthreads();
     if (s_bad) return;  // reported in the error word; nothing was issued
-    if (tid == 0) {
+    if (ROWS) {
+        for (int s = 0; s < kSmStages && s < nplanes; ++s)
+            copy_tile<R>(s_in + s * STAGE_FLOATS, in + (size_t)clampi_s(zfirst + s, 0, nz - 1) * plane, x0, y0, nx, ny,
+                         tid, &bars[s]);
+    } else if (tid == 0) {
         for (int s = 0; s < kSmStages && s < nplanes; ++s) {
             if (s == skip_plane) continue;  // fault injection: this plane's copy is never issued
             mbar_arrive_expect_tx(&bars[s], STAGE_BYTES);
@@ -250,7 +275,7 @@ __global__ void __launch_bounds__(kSmThreads, smooth_min_blocks<R, ZIP>())
     // clamp-to-edge bounds inside the tile (columns / rows that hold real data)
     const int c_lo = max(0, kSmXP - x0), c_hi = min(kSmBW - 1, nx - 1 - (x0 - kSmXP));
     const int r_lo = max(0, R - y0), r_hi = min(IH - 1, ny - 1 - (y0 - R));
-    const bool edge = c_lo > 0 || c_hi < kSmBW - 1 || r_lo > 0 || r_hi < IH - 1;
+    const bool edge = !ROWS && (c_lo > 0 || c_hi < kSmBW - 1 || r_lo > 0 || r_hi < IH - 1);
 
     // x-pass unit of this thread: row xr, outputs 8 xq .. 8 xq + 7
     const bool xunit = tid < 4 * IH;
@@ -283,8 +308,13 @@ __global__ void __launch_bounds__(kSmThreads, smooth_min_blocks<R, ZIP>())
         float2 fpre[2] = {make_float2(0.0f, 0.0f), make_float2(0.0f, 0.0f)};
         if constexpr (ZIP) {
             if (i >= 2 * R) {
-                if (st0) fpre[0] = __ldg(reinterpret_cast<const float2 *>(fp));
-                if (st1) fpre[1] = __ldg(reinterpret_cast<const float2 *>(fp + nx));
+                if constexpr (ROWS) {
+                    if (st0) fpre[0] = make_float2(__ldg(fp), gx + 1 < nx ? __ldg(fp + 1) : 0.0f);
+                    if (st1) fpre[1] = make_float2(__ldg(fp + nx), gx + 1 < nx ? __ldg(fp + nx + 1) : 0.0f);
+                } else {
+                    if (st0) fpre[0] = __ldg(reinterpret_cast<const float2 *>(fp));
+                    if (st1) fpre[1] = __ldg(reinterpret_cast<const float2 *>(fp + nx));
+                }
             }
         }
         const bool ok = mbar_wait(&bars[stage], phase, err, polls);
@@ -302,7 +332,11 @@ __global__ void __launch_bounds__(kSmThreads, smooth_min_blocks<R, ZIP>())
             break;
         }
         // the stage is consumed: refill it with plane i + stages
-        if (tid == 0 && i + kSmStages < nplanes) {
+        if (ROWS) {
+            if (i + kSmStages < nplanes)
+                copy_tile<R>(tile, in + (size_t)clampi_s(zfirst + i + kSmStages, 0, nz - 1) * plane, x0, y0, nx, ny, tid,
+                             &bars[stage]);
+        } else if (tid == 0 && i + kSmStages < nplanes) {
             mbar_arrive_expect_tx(&bars[stage], STAGE_BYTES);
             tma_load_3d(tile, &tmap, x0 - kSmXP, y0 - R, min(max(zfirst + i + kSmStages, 0), nz - 1), &bars[stage]);
         }
@@ -344,7 +378,15 @@ __global__ void __launch_bounds__(kSmThreads, smooth_min_blocks<R, ZIP>())
                         if constexpr (ZIP) {
                             // (first, smoothed) for the voxels gx and gx + 1: one 16-byte store
                             const float2 f = fpre[j];
-                            *reinterpret_cast<float4 *>(o) = make_float4(f.x, acc.x, f.y, acc.y);
+                            if constexpr (ROWS) {
+                                *reinterpret_cast<float2 *>(o) = make_float2(f.x, acc.x);
+                                if (gx + 1 < nx) *reinterpret_cast<float2 *>(o + 2) = make_float2(f.y, acc.y);
+                            } else {
+                                *reinterpret_cast<float4 *>(o) = make_float4(f.x, acc.x, f.y, acc.y);
+                            }
+                        } else if constexpr (ROWS) {
+                            o[0] = acc.x;
+                            if (gx + 1 < nx) o[1] = acc.y;
                         } else {
                             *reinterpret_cast<float2 *>(o) = acc;
                         }
@@ -358,7 +400,9 @@ __global__ void __launch_bounds__(kSmThreads, smooth_min_blocks<R, ZIP>())
             if constexpr (ZIP) fp += plane;
         }
     }
-    if (failed && tid == 0) {
+    if (ROWS) {
+        if (failed) asm volatile("cp.async.wait_all;" ::: "memory");
+    } else if (failed && tid == 0) {
         // drain: wait (bounded) for this CTA's copies still in flight before leaving --
         // planes fail_i .. fail_i + stages - 1 were issued and not consumed
         for (int j = fail_i; j < min(nplanes, fail_i + kSmStages); ++j)
@@ -385,12 +429,14 @@ static int smooth_zchunk(int nx, int ny, int nz, int r)
 
 // The TMA kernel's z chunk: each chunk re-reads 2r halo planes, and CTAs run in waves of
 // `resident` (CTAs per SM x SMs), so pick the number of chunks that minimises
-// waves x (planes per chunk + 2r).  resident <= 0: the plain rule above.
+// waves x (planes per chunk + 2r).  A cube that fills only part of the SMs takes chunks down to
+// r planes: a plane costs a CTA about the same alone or beside two others (64^3, r = 6: 58 us with
+// chunks of 4r = 24 at least, 25 with them; 128^3: 50 and 36).  resident <= 0: the plain rule above.
 static int smooth_zchunk_waves(int nx, int ny, int nz, int r, long long resident)
 {
     if (resident <= 0) return smooth_zchunk(nx, ny, nz, r);
     const long long tiles = (long long)ceil_div(nx, 32) * ceil_div(ny, 32);
-    const int zmin = (4 * r > 16) ? 4 * r : 16;
+    const int zmin = r > 4 ? r : 4;
     long long best = -1;
     int best_zc = nz;
     for (int nch = 1; nch <= nz; ++nch) {
@@ -407,20 +453,20 @@ static int smooth_zchunk_waves(int nx, int ny, int nz, int r, long long resident
     return best_zc;
 }
 
-template <int R, bool ZIP>
+template <int R, bool ZIP, bool ROWS>
 static bool launch_smooth_tma(const float *in, float *out, int nx, int ny, int nz, const SmoothWeights &w,
                               const float *first, cudaStream_t st)
 {
-    CUtensorMap map;
-    if (!encode_tmap_3d_f32(&map, in, nx, ny, nz, kSmBW, kSmTY + 2 * R)) return false;
+    CUtensorMap map{};
+    if (!ROWS && !encode_tmap_3d_f32(&map, in, nx, ny, nz, kSmBW, kSmTY + 2 * R)) return false;
     unsigned *err = device_error_word();
     const size_t smem = smooth_tma_smem<R>();
     if (smem > 48 * 1024)
-        cudaFuncSetAttribute(smooth_tma_kernel<R, ZIP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaFuncSetAttribute(smooth_tma_kernel<R, ZIP, ROWS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     static int per_sm = -1;  // resident CTAs per SM of this instance, queried once
     if (per_sm < 0) {
         int n = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, smooth_tma_kernel<R, ZIP>, kSmThreads, smem) !=
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, smooth_tma_kernel<R, ZIP, ROWS>, kSmThreads, smem) !=
             cudaSuccess) {
             cudaGetLastError();
             n = 0;
@@ -437,7 +483,7 @@ static bool launch_smooth_tma(const float *in, float *out, int nx, int ny, int n
     // SHW_DEBUG_FAULT_TIMEOUT: plane 1 of every chunk is never copied, and waits end after about
     // a millisecond (instead of a second), so every CTA's wait runs out quickly
     const bool fault = debug(SHW_DEBUG_FAULT_TIMEOUT);
-    smooth_tma_kernel<R, ZIP><<<grid, kSmThreads, smem, st>>>(map, out, nx, ny, nz, zc, w, err, first, fault ? 1 : -1,
+    smooth_tma_kernel<R, ZIP, ROWS><<<grid, kSmThreads, smem, st>>>(map, in, out, nx, ny, nz, zc, w, err, first, fault ? 1 : -1,
                                                               fault ? kFaultWaitPolls : kWaitPolls);
     return true;
 }
@@ -460,13 +506,22 @@ template <bool ZIP>
 static shw_status smooth_dispatch(const float *in, float *out, int nx, int ny, int nz, const SmoothWeights &w,
                                   int r, const float *first, cudaStream_t st)
 {
-    // TMA pipeline where its alignment rules hold, the staged kernel otherwise
+    // the pipeline by tensor copies where their alignment rules hold, by row copies elsewhere; the
+    // staged kernel for radius 0, radii above 8, and ragged cubes of few (x, y) blocks at larger
+    // radii, whose short runs of planes pay for the pipeline's unrolled code (67 x 67 x 510, 9
+    // blocks, r = 6: 60 us staged, 80 by row copies; 127^3, 16 blocks: 70 and 44)
     const bool zip_ok = !ZIP || (aligned(first, 8) && aligned(out, 16));
-    if (r >= 1 && r <= 8 && nx % 4 == 0 && aligned(in, 16) && zip_ok && !debug(SHW_DEBUG_SMOOTH_PLAIN)) {
+    // (float2 stores of the tensor-copy form: an 8-byte aligned output)
+    const bool tma = nx % 4 == 0 && aligned(in, 16) && zip_ok && aligned(out, 8);
+    const bool rows = r <= 3 || (long long)ceil_div(nx, kSmTX) * ceil_div(ny, kSmTY) >= 12;
+    if (r >= 1 && r <= 8 && (tma || rows) && !debug(SHW_DEBUG_SMOOTH_PLAIN)) {
         bool ok = false;
         switch (r) {
 #define SHW_T(n) \
-    case n: ok = launch_smooth_tma<n, ZIP>(in, out, nx, ny, nz, w, first, st); break;
+    case n:                                                                             \
+        ok = tma ? launch_smooth_tma<n, ZIP, false>(in, out, nx, ny, nz, w, first, st)  \
+                 : launch_smooth_tma<n, ZIP, true>(in, out, nx, ny, nz, w, first, st);  \
+        break;
             SHW_T(1) SHW_T(2) SHW_T(3) SHW_T(4) SHW_T(5) SHW_T(6) SHW_T(7) SHW_T(8)
 #undef SHW_T
         }
