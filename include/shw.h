@@ -167,8 +167,8 @@ typedef struct {
 
 /* In-ray smoothing of every fetched sample (the cube lookups of Algorithm 1; both cubes
  * for the line ratios).  Reads beyond the cube clamp to the edge voxel like every fetch.
- * Only the general marcher applies it: batch plans and the adjoint reject it
- * (SHW_EUNSUPPORTED). */
+ * The gather and the rolling marcher apply it (equal results): batch plans and the adjoint
+ * reject it (SHW_EUNSUPPORTED). */
 typedef enum {
     SHW_SMOOTH_NONE = 0,
     SHW_SMOOTH_BOX = 1, /* Algorithm 8: (v(p) + sum_{i=1..arm} v(p + i u) + v(p - i u)) / (2 arm + 1),
@@ -330,13 +330,17 @@ shw_status shw_render_backward(const shw_volume *vol, const shw_camera *cam, con
 #define SHW_DEBUG_NO_AXIS_SWEEP 0x1u  /* orthographic spectral-axis views take the general marcher */
 #define SHW_DEBUG_SMOOTH_PLAIN  0x2u  /* smoothing takes its kernel without tensor copies */
 #define SHW_DEBUG_BOX_DIRECT    0x4u  /* in-ray box smoothing by direct fetches, never the lattice sums */
-#define SHW_DEBUG_NO_STAGING    0x8u  /* general views take the gather marcher, not the staged one */
+#define SHW_DEBUG_NO_STAGING    0x8u  /* general views and in-ray smoothing take the gather marcher, not the
+                                         staged or the rolling one */
 #define SHW_DEBUG_FAULT_ALLOC   0x10u /* batch-plan device allocations fail (SHW_ENOMEM) */
 #define SHW_DEBUG_FAULT_GRAPH   0x20u /* batch-plan graph capture fails (SHW_ECUDA) */
 #define SHW_DEBUG_REQUIRE_STAGING 0x80u /* a render of a float32 cube or pair storage that neither the
-                                           spectral-axis sweep nor the staged marcher serves is
-                                           refused (SHW_EUNSUPPORTED) instead of taking the gather
-                                           marcher */
+                                           spectral-axis sweep nor the staged marcher serves, or an
+                                           in-ray smoothing of one float32 cube that the rolling
+                                           marcher does not, is refused (SHW_EUNSUPPORTED) instead of
+                                           taking the gather marcher; and the sweep, the staged and
+                                           the rolling marcher serve what they can, also where
+                                           gathering would be faster */
 #define SHW_DEBUG_FAULT_TIMEOUT 0x40u /* smoothing launched while set (its tensor-copy form: radius 1..8,
                                          nx a multiple of 4) leaves the copy of each z chunk's second
                                          plane unissued and bounds its waits at about 1 ms: every CTA

@@ -491,7 +491,7 @@ struct SlabRing {
 // cells from the current cell; the thickest whose staged box fits a stage wins (one cell,
 // its box clipped to a stage, when none fits), and empty runs are skipped.  False if a
 // wait gave up.
-template <class EP, int M>
+template <class EP, int M, bool EARLY>
 __device__ __forceinline__ bool produce_tile(const TileRays &r, bool persp, const CUtensorMap *map_n,
                                              const CUtensorMap *map_w, const RenderArgs &a, int tile, int seq,
                                              unsigned char *stages, SlabRing &ring)
@@ -511,7 +511,7 @@ __device__ __forceinline__ bool produce_tile(const TileRays &r, bool persp, cons
             hi_c = min(hi_c, e);
     }
     int cur = dir > 0 ? lo_c : hi_c;
-    while (cur >= lo_c && cur <= hi_c && !tile_dead(ring.sh.dead, seq)) {
+    while (cur >= lo_c && cur <= hi_c && !(EARLY && tile_dead(ring.sh.dead, seq))) {
         const int len = lane + 1;
         const int c0 = dir > 0 ? cur : max(cur - len + 1, lo_c);
         const int c1 = dir > 0 ? min(cur + len - 1, hi_c) : cur;
@@ -559,7 +559,7 @@ __device__ __forceinline__ bool produce_tile(const TileRays &r, bool persp, cons
 // The producer warp: takes tiles from the counter and stages, for each, the slabs its rays
 // cross, front to back.  Every stage carries a header: a tile's start, one slab, a tile's
 // end, or the end of the launch.
-template <class EP>
+template <class EP, bool EARLY>
 __device__ void slab_producer(const CUtensorMap *maps, const shw_camera &cam, const RenderArgs &a, const SlabArgs &sa,
                               unsigned char *stages, SlabShared &sh)
 {
@@ -581,11 +581,11 @@ __device__ void slab_producer(const CUtensorMap *maps, const shw_camera &cam, co
         const bool persp = !cam.ortho;
         // maps: x-major; y-major narrow, wide; z-major narrow, wide
         if (r.major == 0)
-            ok = produce_tile<EP, 0>(r, persp, &maps[0], &maps[0], a, (int)t, seq, stages, ring);
+            ok = produce_tile<EP, 0, EARLY>(r, persp, &maps[0], &maps[0], a, (int)t, seq, stages, ring);
         else if (r.major == 1)
-            ok = produce_tile<EP, 1>(r, persp, &maps[1], &maps[2], a, (int)t, seq, stages, ring);
+            ok = produce_tile<EP, 1, EARLY>(r, persp, &maps[1], &maps[2], a, (int)t, seq, stages, ring);
         else
-            ok = produce_tile<EP, 2>(r, persp, &maps[3], &maps[4], a, (int)t, seq, stages, ring);
+            ok = produce_tile<EP, 2, EARLY>(r, persp, &maps[3], &maps[4], a, (int)t, seq, stages, ring);
         if (ok) ok = ring.post_plain(kStageTileEnd, (int)t);
     }
     // the CTA may not exit while a tensor copy into its shared memory is in flight: wait
@@ -699,7 +699,8 @@ __device__ void slab_consumer(const S &s, const shw_camera &cam, const RenderArg
             has = false;
         }
         __syncwarp();
-        if (h.type != kStageTileEnd) report_dead(sh.dead, seq, live && k < kb, said);
+        if constexpr (is_composite<MODE>)  // (the other modes take every sample)
+            if (h.type != kStageTileEnd) report_dead(sh.dead, seq, live && k < kb, said);
         if (lane == 0) mbar_arrive(&sh.empty[si]);
     }
 }
@@ -728,7 +729,7 @@ __global__ void __launch_bounds__(kSlabThreads, kSlabMinBlocks)
     }
     __syncthreads();
     if ((threadIdx.x >> 5) == kSlabWarps)
-        slab_producer<EP>(maps.m, cam, a, sa, stages, sh);
+        slab_producer<EP, is_composite<MODE>>(maps.m, cam, a, sa, stages, sh);
     else
         slab_consumer<MODE, EP>(s, cam, a, sa, stages, sh);
 }
