@@ -991,10 +991,15 @@ shw_status launch_render_modes(int mode, int interp, const S &s, const S &s2, co
     // image of only a few tiles per CTA takes fewer of the raised counts, down to 8 per SM: more would leave
     // nothing to even out the long rays with (128^3 on 500 x 500, compositing: 137 us with 8 per
     // SM, 193 with 12; 1000 x 1000: 389 and 383).  Nearest sampling's rays are too short to
-    // mind (45 us with 11 per SM, 53 with 8).
+    // mind (45 us with 11 per SM, 53 with 8).  Compositing a cube of more than 2^29 voxels also
+    // stays at 8: more rays in flight than that draw their planes from HBM over and over (1024^3 on
+    // 1000 x 1000, clipped, gathered: 14.1 ms with 12 per SM, 6.6 with 8 at yaw 60, though 3.1 and
+    // 4.3 along z; 641^3: 3.1 and 2.7, 1.9 and 2.4).
     auto persistent = [&](auto kern, int per_sm, bool more_ctas) {
         long long g = std::min<long long>((long long)per_sm * nsm, tiles);
         if (SMK == 0 && interp != SHW_NEAREST && more_ctas) g = std::min(g, std::max(tiles / 4, 8LL * nsm));
+        if (SMK == 0 && interp != SHW_NEAREST && more_ctas && (double)s.nx * s.ny * s.nz > 536870912.0)
+            g = std::min(g, 8LL * nsm);
         kern<<<(unsigned)std::max<long long>(g, 1), block, 0, st>>>(s, s2, cam, a, ctr, nwarp_tiles);
     };
     if (SMK > 0 && (ctr == nullptr || nsm <= 0)) return SHW_ECUDA;

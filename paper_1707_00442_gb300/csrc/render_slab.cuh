@@ -772,11 +772,19 @@ shw_status slab_launch_one(const SlabMaps &maps, const S &s, const shw_camera &c
 //     (200^3 on 400 x 400, yaw 85: 344 against 180).  A cube larger than the second-level cache
 //     is gathered from HBM, and a footprint up to 50 cells wide still stages better (512^3 on
 //     640 x 640: 816 against 1298; the pair storage of 512^3 on 1000 x 1000, yaw 70: 2693
-//     against 3835);
+//     against 3835).  The less of the cube that cache holds, the more a gather costs, so the
+//     limit grows by 24 cells for each doubling above 2^27 voxels, up to 100: at 70 to 80 cells
+//     and 2^28 voxels (512 x 512 x 1024 on 1000 x 1000, yaw 70) MIP takes 2083 us staged and
+//     4054 gathered, but with 134M voxels and 110 cells (512^3 on 400 x 400, yaw 90) gathering
+//     is 1.6 times as fast; 1024^3 on 1000 x 1000, yaw 70 (95 cells): 5831 against 7750, on
+//     700 x 700, yaw 90 (121 cells) gathering is 1.3 times as fast;
 //   - above a fifth of a voxel per pixel: below, the gathers hit the first-level cache and the
 //     stages' hand-overs cost more (64^3 on 1000 x 1000, compositing: 267 against 217).
 // Over 700 renders (48^3 .. 512^3 and oblong cubes, 128^2 .. 1000^2, five views, MIP and
-// compositing) the rule is 2 % from the better of the two on average, always staging 21 %.
+// compositing) the rule is 2 % from the better of the two on average, always staging 21 %;
+// over 584 renders of cubes above the cache's size (400^3 .. 1024^3, float32 and pairs, 250^2 ..
+// 2000^2, eight views) 4.3 % on average (early ends that compositing meets are not foreseen),
+// always staging 16 %, a limit of 50 cells 6.6 %.
 template <class G>
 inline bool slab_pays(const shw_camera &c, int nx, int ny, int nz)
 {
@@ -810,8 +818,10 @@ inline bool slab_pays(const shw_camera &c, int nx, int ny, int nz)
             ext[k] = fminf(hi - lo + 2.0f, (float)(k == 0 ? na : nb));
         }
         if (M == 0) return ceilf(ext[0] / kSlabRows) * kSlabRows * ext[1] * G::kBXx <= 0.75f * G::kStageElems;
-        const bool hbm = (double)nx * ny * nz * G::kBytes > 128e6;
-        return ext[0] <= (hbm ? 50.0f : (float)(G::kBXw - 2)) &&
+        const float vox = (float)nx * (float)ny * (float)nz;
+        const bool hbm = vox * (float)G::kBytes > 128e6f;
+        const float widest = fminf(fmaxf(50.0f + 24.0f * (log2f(vox) - 27.0f), 50.0f), 100.0f);
+        return ext[0] <= (hbm ? widest : (float)(G::kBXw - 2)) &&
                2.0f * ext[1] * (float)(ext[0] + 3.0f <= G::kBXn ? G::kBXn : G::kBXw) <= (float)G::kStageElems;
     };
     if (r.major == 0) return fits(std::integral_constant<int, 0>{}, ny, nz, nx);
