@@ -197,7 +197,7 @@ struct RollRing {
             RollHdr h{};
             h.type = type;
             h.tile = tile;
-            h.m0 = seq;
+            h.m0 = seq % kDeadSlots;
             if (type == kStageTile) sh.dead[seq % kDeadSlots] = 0;
             sh.hdr[st] = h;
             mbar_arrive(&sh.full[st]);
@@ -666,8 +666,8 @@ __device__ __forceinline__ void roll_consumer(const S &s, const shw_camera &cam,
     RayFx r;
     long long pix = 0;
     int N = 0;
-    bool has = false, live = false, said = false;
-    int seq = 0;
+    bool has = false, live = false;
+    int slot = -1;  // the tile's entry of sh.dead
     for (int posts = 0;; ++posts) {
         const int si = posts % kRollBars;
         if (!slab_wait(&sh.full[si], (uint32_t)((posts / kRollBars) & 1), quit, ra.err, ra.polls)) return;
@@ -682,8 +682,7 @@ __device__ __forceinline__ void roll_consumer(const S &s, const shw_camera &cam,
             const bool hit = has && !quick_miss(cam, px, py, s.nx, s.ny, s.nz) &&
                              setup_ray(cam, px, py, s.nx, s.ny, s.nz, a.step, r);
             N = hit ? min(r.N, a.nmax) : 0;
-            seq = h.m0;
-            said = false;
+            slot = h.m0;
             live = N > 0;
             q.st = typename RollMarch<MODE, KIND>::St{};
             q.done = 0;
@@ -734,7 +733,7 @@ __device__ __forceinline__ void roll_consumer(const S &s, const shw_camera &cam,
             has = false;
         }
         __syncwarp();
-        if (h.type != kStageTileEnd) report_dead(sh.dead, seq, live && q.k < q.kend, said);
+        if (h.type != kStageTileEnd) report_dead(sh.dead, slot, live && q.k < q.kend);
         if (lane == 0) mbar_arrive(&sh.empty[si]);
     }
 }

@@ -444,12 +444,12 @@ __device__ __forceinline__ bool tile_dead(const int *dead, int seq)
     return __shfl_sync(0xffffffffu, d, 0) == kSlabWarps;
 }
 
-// A consumer warp's report, once per tile (`said`): no lane needs another slab.
-__device__ __forceinline__ void report_dead(int *dead, int seq, bool need, bool &said)
+// A consumer warp's report, once per tile (`slot` is then -1): no lane needs another slab.
+__device__ __forceinline__ void report_dead(int *dead, int &slot, bool need)
 {
-    if (!said && !__any_sync(0xffffffffu, need)) {
-        said = true;
-        if ((threadIdx.x & 31) == 0) atomicAdd(dead + seq % kDeadSlots, 1);
+    if (slot >= 0 && !__any_sync(0xffffffffu, need)) {
+        if ((threadIdx.x & 31) == 0) atomicAdd(dead + slot, 1);
+        slot = -1;
     }
 }
 
@@ -467,7 +467,7 @@ struct SlabRing {
             return -1;
         return st;
     }
-    // a stage that carries only its header (a tile's start: and the tile's number in this CTA)
+    // a stage that carries only its header (a tile's start: and its entry of sh.dead)
     __device__ __forceinline__ bool post_plain(int type, int tile, int seq = 0)
     {
         const int st = take();
@@ -476,7 +476,7 @@ struct SlabRing {
             SlabHdr h{};
             h.type = type;
             h.tile = tile;
-            h.s_lo = seq;
+            h.s_lo = seq % kDeadSlots;
             if (type == kStageTile) sh.dead[seq % kDeadSlots] = 0;
             sh.hdr[st] = h;
             mbar_arrive(&sh.full[st]);
@@ -619,8 +619,8 @@ __device__ void slab_consumer(const S &s, const shw_camera &cam, const RenderArg
     CacheOf<S> cc;
     long long X = 0, Y = 0, Z = 0, pix = 0;
     int N = 0, k = 0, kb = 0, done = 0;
-    bool has = false, live = false, said = false;
-    int seq = 0;
+    bool has = false, live = false;
+    int slot = -1;  // the tile's entry of sh.dead
     for (int posts = 0;; ++posts) {
         const int si = posts % kSlabStages;
         if (!slab_wait(&sh.full[si], (uint32_t)((posts / kSlabStages) & 1), quit, sa.err, sa.polls)) return;
@@ -637,8 +637,7 @@ __device__ void slab_consumer(const S &s, const shw_camera &cam, const RenderArg
             N = hit ? min(r.N, a.nmax) : 0;
             st = St{};
             done = 0;
-            seq = h.s_lo;
-            said = false;
+            slot = h.s_lo;
             live = N > 0;
             if (live) {
                 int ka;
@@ -700,7 +699,7 @@ __device__ void slab_consumer(const S &s, const shw_camera &cam, const RenderArg
         }
         __syncwarp();
         if constexpr (is_composite<MODE>)  // (the other modes take every sample)
-            if (h.type != kStageTileEnd) report_dead(sh.dead, seq, live && k < kb, said);
+            if (h.type != kStageTileEnd) report_dead(sh.dead, slot, live && k < kb);
         if (lane == 0) mbar_arrive(&sh.empty[si]);
     }
 }
