@@ -849,9 +849,10 @@ inline bool roll_geometry(const shw_camera &cam, const int n[3], int H, bool tma
         if (wa[M] <= 0 || wb[M] <= 0) continue;  // no sampled tile takes this axis: none will
         const int A = M == 0 ? 1 : 0, B = M == 2 ? 1 : 2;
         G.g = M == 0 ? kRollXG : 1;
-        // room for the tiles and planes between the sampled ones
-        G.wb = std::min(wb[M] + 2 + (wb[M] - 2 * H) / 10, n[B]);
-        G.wa = std::min(wa[M] + 2 + (wa[M] - 2 * H) / 10, n[A]);
+        // room for the tiles and planes between the sampled ones (a footprint that the cube clips
+        // may be narrower than the taps' reach)
+        G.wb = std::min(wb[M] + 2 + std::max(wb[M] - 2 * H, 0) / 10, n[B]);
+        G.wa = std::min(wa[M] + 2 + std::max(wa[M] - 2 * H, 0) / 10, n[A]);
         int pad = 0;
         if (M != 0 && tmaps) {
             G.sb = G.wa = roll_pitch(G.wa + 3, ext[M], 0);  // a tensor copy's rows; its x start on 16 bytes
