@@ -769,9 +769,10 @@ shw_status launch_axis(int mode, int interp, bool up, const CUtensorMap &map, co
 {
 #define SHW_AX(M, I, U)                                                                                 \
     do {                                                                                                \
-        /* static + dynamic shared memory may pass the 48 KB default: always opt in */                \
+        /* static + dynamic shared memory may pass the 48 KB default: always opt in, and to one size  \
+           (the limit is the kernel's: a concurrent call must not lower it) */                         \
         cudaFuncSetAttribute(axis_kernel<M, I, U, FIX>, cudaFuncAttributeMaxDynamicSharedMemorySize,   \
-                             (int)smem);                                                                \
+                             kAxSmemLimit);                                                             \
         axis_kernel<M, I, U, FIX><<<grid, AxCfg<axis_warps<M>()>::threads, smem, st>>>(map, data, c, a, A);  \
     } while (0)
 #define SHW_AXI(M, I)           \

@@ -885,7 +885,10 @@ shw_status roll_launch_one(const RollMaps &maps, const S &s, const shw_camera &c
                            const RollArgs &ra, size_t smem, cudaStream_t st)
 {
     auto kern = roll_kernel<MODE, KIND, S>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+    // The limit is the kernel's, shared by every thread of the process: always the largest ring, so
+    // that no concurrent call lowers it between another's setting and launch.  (Residency follows
+    // from the launch's own size.)
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kRollBudget1) != cudaSuccess) {
         cudaGetLastError();
         return SHW_ECUDA;
     }
