@@ -36,10 +36,6 @@ shw_status render_axis(int mode, int interp, const shw_volume &v, const shw_came
     const double ext_x = (kAxTX - 1) * std::fabs(ax) + (kAxTY - 1) * std::fabs(bx);
     const double ext_y = (kAxTX - 1) * std::fabs(ay) + (kAxTY - 1) * std::fabs(by);
     AxisArgs A{};
-    // the tile's footprint plus margins: 2 voxels each side for FP32 rounding of the box
-    // corner and the interpolation neighbour, and up to 3 to align the x start to 16 bytes
-    A.bw = ((int)std::ceil(ext_x) + 8 + 3) & ~3;
-    A.bh = (int)std::ceil(ext_y) + 6;
     // rows that no tensor copy takes: row copies, with 32-bit element indexes.  A few planes under
     // a small image are gathered as fast (71 x 71 x 48 on 71^2: 48 us gathered, 52 by row copies;
     // 67 x 67 x 193 on 134^2: 137 and 121, 601 x 601 x 300 on 601^2: 961 and 494)
@@ -47,20 +43,11 @@ shw_status render_axis(int mode, int interp, const shw_volume &v, const shw_came
     if (A.rows && ((long long)v.nx * v.ny * v.nz >= (1ll << 31) ||
                    (v.nz < 96 && (long long)c.width * c.height < 65536 && !debug(SHW_DEBUG_REQUIRE_STAGING))))
         return SHW_EUNSUPPORTED;
-    const bool fix = A.bw <= kFixBW && A.bh <= kFixBH && !A.rows;
-    if (fix) {
-        A.bw = kFixBW;
-        A.bh = kFixBH;
-    }
-    if (A.bw > 256 || A.bh > 256) return SHW_EUNSUPPORTED;  // the tensor copy's box limit
-    // (a row copy brings whole 16-byte pieces, up to 10 floats more than the box)
-    A.pitch = A.rows ? A.bw + 10 + ((v.nx - A.bw - 10) & 3) : A.bw;
     A.goff = (int)((reinterpret_cast<uintptr_t>(v.data) >> 2) & 3);
-    // TMA destinations start on 128 bytes
-    A.stage_stride = fix ? kFixStride : (A.pitch * A.bh + (A.rows ? 16 : 0) + 31) & ~31;
     const int kmode = (mode == SHW_MIP && a.index == nullptr) ? kMipValue : mode;
-    const size_t smem = (size_t)axis_stages(kmode, fix) * A.stage_stride * 4;
-    if (smem > (size_t)kAxSmemLimit) return SHW_EUNSUPPORTED;
+    bool fix;
+    size_t smem;
+    if (!axis_box(ext_x, ext_y, v.nx, kmode, A, fix, smem)) return SHW_EUNSUPPORTED;
     A.nx = v.nx;
     A.ny = v.ny;
     A.nz = v.nz;

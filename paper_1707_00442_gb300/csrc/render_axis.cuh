@@ -759,6 +759,30 @@ __global__ void __launch_bounds__(AxCfg<W>::threads, MODE == SHW_COMPOSITE ? 1 :
     }
 }
 
+// The staged box of a tile whose pixels span ext_x x ext_y voxels (A.rows set): its extents, row
+// pitch, stage stride, whether the fixed box serves it, and the ring's bytes.  False: no box that
+// fits the copies and the shared memory.
+inline bool axis_box(double ext_x, double ext_y, int nx, int mode, AxisArgs &A, bool &fix, size_t &smem)
+{
+    if (!(ext_x <= 256.0 && ext_y <= 256.0)) return false;  // (also before the conversions to int)
+    // the tile's footprint plus margins: 2 voxels each side for FP32 rounding of the box
+    // corner and the interpolation neighbour, and up to 3 to align the x start to 16 bytes
+    A.bw = ((int)std::ceil(ext_x) + 8 + 3) & ~3;
+    A.bh = (int)std::ceil(ext_y) + 6;
+    fix = A.bw <= kFixBW && A.bh <= kFixBH && !A.rows;
+    if (fix) {
+        A.bw = kFixBW;
+        A.bh = kFixBH;
+    }
+    if (A.bw > 256 || A.bh > 256) return false;  // the tensor copy's box limit
+    // (a row copy brings whole 16-byte pieces, up to 10 floats more than the box)
+    A.pitch = A.rows ? A.bw + 10 + ((nx - A.bw - 10) & 3) : A.bw;
+    // TMA destinations start on 128 bytes
+    A.stage_stride = fix ? kFixStride : (A.pitch * A.bh + (A.rows ? 16 : 0) + 31) & ~31;
+    smem = (size_t)axis_stages(mode, fix) * A.stage_stride * 4;
+    return smem <= (size_t)kAxSmemLimit;
+}
+
 // Launch the sweep for one (mode, interp, direction); FIX selects the fixed box.
 // mode may be kMipValue.  Returns SHW_EUNSUPPORTED for a mode it has no kernel for.
 // Instantiated once per FIX, each in its own translation unit.
