@@ -177,7 +177,8 @@ __global__ void __launch_bounds__(kBwdThreads) backward_kernel(SamplerF32<Idx> s
                 const float gcr = g.x * wc, gcg = g.y * wc, gcb = g.z * wc;
                 if (on) gT = gT * (1.0f - al) + al * gc;
                 const float galpha = (on && alpha >= 0.0f && alpha <= 1.0f) ? ga : 0.0f;
-                gs = __fmaf_rn(galpha, c.w, gs);
+                // (an idle lane's c is the map at DATAMIN, which no sample need read: 0 * c.w may be NaN)
+                if (on) gs = __fmaf_rn(galpha, c.w, gs);
                 const float gca = galpha * a.opacity_scale;
                 if (a.grad_lut != nullptr) {
                     // lanes on the same entry take turns (a lane without a sample has an entry of its own)

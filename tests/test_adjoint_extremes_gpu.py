@@ -1,0 +1,44 @@
+"""The adjoint at the ends of its input range on the GPU: colour maps with non-finite entries that no
+sample reads, gradients that overflow, checkpoints with rays that took no sample.  Each is compared
+with a run on ordinary values of the same shape, so only what must be unaffected is asserted."""
+import numpy as np
+import pytest
+import torch
+
+import scene
+from parity import shw, to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def m():
+    return shw()
+
+
+def _backward(m, cube, cam, lut, g, scale, edit=None, **kw):
+    out = m.render(cube, cam, "composite", lut=lut, opacity_scale=scale, ckpt=True, **kw)
+    if edit is not None:
+        edit(out["ckpt"])
+    gv, gl, gs = torch.zeros_like(cube), torch.zeros_like(lut), torch.zeros(1, device="cuda")
+    m.render_backward(cube, cam, g, out["ckpt"], lut=lut, opacity_scale=scale, grad_vol=gv, grad_lut=gl, grad_scale=gs, **kw)
+    m.sync_status()
+    return gv, gl, float(gs.item())
+
+
+@pytest.mark.parametrize("interp", ["trilinear", "nearest"])
+@pytest.mark.parametrize("value", [np.nan, np.inf])
+def test_knots_that_no_sample_reads(m, interp, value):
+    """Voxels in [0.25, 0.75] of the domain [0, 1] read knots 63 to 192: knots 0 and 1 may hold anything."""
+    dims = (24, 20, 28)
+    cube = 0.25 + 0.5 * torch.rand(dims[::-1], generator=torch.Generator("cuda").manual_seed(3), device="cuda")
+    cam = scene.orbit_camera(dims, 30, 20, 50, 41)  # rays of different lengths in every warp
+    g = torch.rand((41, 50, 4), generator=torch.Generator("cuda").manual_seed(4), device="cuda")
+    lut = to_dev(scene.linear_lut())
+    bad = lut.clone()
+    bad[:2] = value
+    kw = dict(lo=0.0, hi=1.0, interp=interp)
+    _, _, want = _backward(m, cube, cam, lut, g, 0.05, **kw)
+    gv, gl, gs = _backward(m, cube, cam, bad, g, 0.05, **kw)
+    assert bool(torch.isfinite(gv).all()) and bool(torch.isfinite(gl).all())
+    assert gs == pytest.approx(want, rel=1e-4)  # (the sums' order varies)
