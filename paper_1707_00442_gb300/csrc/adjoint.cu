@@ -227,7 +227,7 @@ __global__ void __launch_bounds__(kBwdThreads) backward_kernel(SamplerF32<Idx> s
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) gs += __shfl_xor_sync(0xffffffffu, gs, o);
         const float y = __fsub_rn(gs, gs_comp), z = __fadd_rn(gs_sum, y);
-        gs_comp = __fsub_rn(__fsub_rn(z, gs_sum), y);
+        gs_comp = isfinite(z) ? __fsub_rn(__fsub_rn(z, gs_sum), y) : 0.0f;  // (an infinite sum stays infinite)
         gs_sum = z;
     }
     // the scale gradient: one shared atomic per warp; the colour map's: the warps' sums of an

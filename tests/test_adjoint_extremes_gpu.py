@@ -42,3 +42,17 @@ def test_knots_that_no_sample_reads(m, interp, value):
     gv, gl, gs = _backward(m, cube, cam, bad, g, 0.05, **kw)
     assert bool(torch.isfinite(gv).all()) and bool(torch.isfinite(gl).all())
     assert gs == pytest.approx(want, rel=1e-4)  # (the sums' order varies)
+
+
+def test_scale_gradient_that_overflows(m):
+    """One pixel at the image's centre (the first tile that any warp takes; the image has more tiles than
+    the device has warps) whose gradients overflow: the sum is infinite, not NaN."""
+    dims = (24, 24, 24)
+    cube = 0.25 + 0.5 * torch.rand(dims, generator=torch.Generator("cuda").manual_seed(3), device="cuda")
+    cam = scene.orbit_camera(dims, 0, 0, 640, 640)
+    lut = to_dev(scene.linear_lut())
+    g = torch.zeros((640, 640, 4), device="cuda")
+    g[..., 3] = 1.0
+    g[320, 320, 3] = 3e38  # times 20 and more samples' alpha
+    _, _, gs = _backward(m, cube, cam, lut, g, 0.05, lo=0.0, hi=1.0)
+    assert gs == np.inf
