@@ -131,7 +131,7 @@ __global__ void __launch_bounds__(kBwdThreads) backward_kernel(SamplerF32<Idx> s
         const long long pix = inside ? (long long)py * a.width + px : 0;
         RayFx r;
         const bool hit = inside && setup_ray(cam, px, py, s.nx, s.ny, s.nz, a.step, r);
-        const int K = hit ? min(min(a.ckpt_K[pix], r.N), a.nmax) : 0;
+        const int K = hit ? max(min(min(a.ckpt_K[pix], r.N), a.nmax), 0) : 0;
         const float4 g = hit ? a.grad_rgba[pix] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         float gT = -g.w;  // alpha_out = 1 - T_K
         float gs = 0.0f;

@@ -56,3 +56,23 @@ def test_scale_gradient_that_overflows(m):
     g[320, 320, 3] = 3e38  # times 20 and more samples' alpha
     _, _, gs = _backward(m, cube, cam, lut, g, 0.05, lo=0.0, hi=1.0)
     assert gs == np.inf
+
+
+def test_checkpoints_without_samples(m):
+    """A checkpoint whose count for some pixels is zero or negative: those rays give nothing, and the
+    others what they gave."""
+    dims = (24, 20, 28)
+    cube = 0.25 + 0.5 * torch.rand(dims[::-1], generator=torch.Generator("cuda").manual_seed(3), device="cuda")
+    cam = scene.orbit_camera(dims, 30, 20, 50, 41)
+    lut = to_dev(scene.linear_lut())
+    g = torch.rand((41, 50, 4), generator=torch.Generator("cuda").manual_seed(4), device="cuda")
+
+    def counts(value):
+        def edit(ckpt):
+            ckpt[:4 * 41 * 50].view(torch.int32)[7::13] = value
+        return edit
+
+    zero, negative = (_backward(m, cube, cam, lut, g, 0.05, edit=counts(v), lo=0.0, hi=1.0) for v in (0, -1))
+    for a, b in zip(zero[:2], negative[:2]):
+        assert float(a.abs().max()) > 0 and torch.allclose(a, b, rtol=1e-4, atol=1e-6 * float(a.abs().max()))
+    assert zero[2] != 0.0 and negative[2] == pytest.approx(zero[2], rel=1e-4)
