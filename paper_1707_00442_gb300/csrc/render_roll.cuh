@@ -93,7 +93,7 @@ struct RollShared {
     // cell c of a step: the lateral cells [x, x + y) along A and [z, z + w) along B whose
     // corners and taps the planes of its window all hold
     int4 range[kRollTable];
-    int dead[kDeadSlots];  // (SlabShared)
+    int done[kSlabWarps];  // (SlabShared)
     int quit;
     int pad[3];
 };
@@ -189,7 +189,7 @@ struct RollRing {
                 return false;
         return true;
     }
-    __device__ __forceinline__ bool post_plain(int type, int tile, int seq = 0)
+    __device__ __forceinline__ bool post_plain(int type, int tile)
     {
         if (!drain_to(posts - kRollBars)) return false;
         const int st = posts % kRollBars;
@@ -197,8 +197,6 @@ struct RollRing {
             RollHdr h{};
             h.type = type;
             h.tile = tile;
-            h.m0 = seq % kDeadSlots;
-            if (type == kStageTile) sh.dead[seq % kDeadSlots] = 0;
             sh.hdr[st] = h;
             mbar_arrive(&sh.full[st]);
         }
@@ -285,7 +283,7 @@ __device__ __forceinline__ void roll_xplanes(const RollArgs &ra, const RollGeom 
 
 template <int M>
 __device__ __forceinline__ bool roll_produce(const TileRays &r, bool persp, const CUtensorMap *map,
-                                             const RenderArgs &a, const RollArgs &ra, int tile, int seq, float *stage,
+                                             const RenderArgs &a, const RollArgs &ra, int tile, float *stage,
                                              RollRing &ring)
 {
     using AX = RollAxes<M>;
@@ -323,8 +321,8 @@ __device__ __forceinline__ bool roll_produce(const TileRays &r, bool persp, cons
     const int before = ring.posts - 2;  // the last post before this tile's start: it may read the ring
     bool fresh = true;
     int have_lo = 0, have_hi = -1;  // slots staged
-    for (int m0 = floor_div(dir > 0 ? first : last, s) * s; (dir > 0 ? m0 <= last : m0 + s > first) && !tile_dead(sh.dead, seq);
-         m0 += dir * s) {
+    for (int m0 = floor_div(dir > 0 ? first : last, s) * s; dir > 0 ? m0 <= last : m0 + s > first; m0 += dir * s) {
+        if (tile_done(sh.done, tile)) break;  // every ray of the tile has ended
         const int plo = max(m0 - H, 0), phi = min(m0 + s + H, n_m - 1);
         const int slo = plo / g, shi = phi / g;
         const int c0 = fresh ? slo : (dir > 0 ? have_hi + 1 : slo), c1 = fresh ? shi : (dir > 0 ? shi : have_lo - 1);
@@ -425,7 +423,7 @@ __device__ __forceinline__ void roll_producer(const CUtensorMap *maps, const shw
     RollRing ring{sh, ra};
     const int on[3] = {ra.geo[0].on, ra.geo[1].on, ra.geo[2].on};
     bool ok = true;
-    for (int seq = 0; ok; ++seq) {
+    while (ok) {
         unsigned t = 0;
         if (lane == 0) t = atomicAdd(ra.ctr, 1u);
         t = __shfl_sync(0xffffffffu, t, 0);
@@ -433,17 +431,17 @@ __device__ __forceinline__ void roll_producer(const CUtensorMap *maps, const shw
             ring.post_plain(kStageExit, 0);
             break;
         }
-        if (!ring.post_plain(kStageTile, (int)t, seq)) break;
+        if (!ring.post_plain(kStageTile, (int)t)) break;
         int tx, ty;
         slab_tile((int)t, a, tx, ty);
         const TileRays r = roll_rays(cam, tx * kSlabTW, ty * kSlabTH, on, ra.xbias);
         const bool persp = !cam.ortho;
         if (r.major == 0)
-            ok = roll_produce<0>(r, persp, nullptr, a, ra, (int)t, seq, stage, ring);
+            ok = roll_produce<0>(r, persp, nullptr, a, ra, (int)t, stage, ring);
         else if (r.major == 1)
-            ok = roll_produce<1>(r, persp, &maps[0], a, ra, (int)t, seq, stage, ring);
+            ok = roll_produce<1>(r, persp, &maps[0], a, ra, (int)t, stage, ring);
         else
-            ok = roll_produce<2>(r, persp, &maps[1], a, ra, (int)t, seq, stage, ring);
+            ok = roll_produce<2>(r, persp, &maps[1], a, ra, (int)t, stage, ring);
         if (ok) ok = ring.post_plain(kStageTileEnd, (int)t);
     }
     // no exit while a copy into this CTA's shared memory is in flight: wait (bounded) for the
@@ -667,7 +665,6 @@ __device__ __forceinline__ void roll_consumer(const S &s, const shw_camera &cam,
     long long pix = 0;
     int N = 0;
     bool has = false, live = false;
-    int slot = -1;  // the tile's entry of sh.dead
     for (int posts = 0;; ++posts) {
         const int si = posts % kRollBars;
         if (!slab_wait(&sh.full[si], (uint32_t)((posts / kRollBars) & 1), quit, ra.err, ra.polls)) return;
@@ -682,7 +679,6 @@ __device__ __forceinline__ void roll_consumer(const S &s, const shw_camera &cam,
             const bool hit = has && !quick_miss(cam, px, py, s.nx, s.ny, s.nz) &&
                              setup_ray(cam, px, py, s.nx, s.ny, s.nz, a.step, r);
             N = hit ? min(r.N, a.nmax) : 0;
-            slot = h.m0;
             live = N > 0;
             q.st = typename RollMarch<MODE, KIND>::St{};
             q.done = 0;
@@ -733,7 +729,7 @@ __device__ __forceinline__ void roll_consumer(const S &s, const shw_camera &cam,
             has = false;
         }
         __syncwarp();
-        if (h.type != kStageTileEnd) report_dead(sh.dead, slot, live && q.k < q.kend);
+        report_done(sh.done, sh.hdr[si].tile, live && q.k < q.kend);
         if (lane == 0) mbar_arrive(&sh.empty[si]);
     }
 }
@@ -753,6 +749,7 @@ __global__ void __launch_bounds__(kSlabThreads, kRollMinBlocks)
             mbar_init(&sh.full[i], 1);
             mbar_init(&sh.empty[i], kSlabWarps);
         }
+        for (int w = 0; w < kSlabWarps; ++w) sh.done[w] = -1;
         sh.quit = 0;
         fence_barrier_init();
     }

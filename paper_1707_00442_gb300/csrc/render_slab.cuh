@@ -425,32 +425,30 @@ struct SlabArgs {
     int polls;      // bound of every wait (sleeping polls)
 };
 
-// dead[t % 4]: consumer warps none of whose rays needs another slab of the CTA's t-th tile (all
-// have stopped or passed the interior).  The producer ends the tile when all are; a hint, so
+// done[w]: the last tile in which consumer warp w needs no further slab (all its rays have stopped
+// or passed the interior).  The producer ends a tile when every warp's entry names it; a hint, so
 // plain shared-memory accesses do.  (Compositing 512^3 on 1000 x 1000 at opacity scale 0.22, whose
 // rays stop within a few dozen samples: 576 us with every tile staged to its far end, 326 with it.)
-constexpr int kDeadSlots = 4;  // a slot is zeroed when the tiles before the last have been consumed
 struct SlabShared {
     SlabHdr hdr[kSlabStages];
     uint64_t full[kSlabStages], empty[kSlabStages];
-    int dead[kDeadSlots];
+    int done[kSlabWarps];
     int quit;
 };
 
-// Whether every consumer warp is done with tile number `seq` (one value for the whole warp).
-__device__ __forceinline__ bool tile_dead(const int *dead, int seq)
+// Whether every consumer warp is done with `tile` (one value for the whole producer warp).
+__device__ __forceinline__ bool tile_done(const int *done, int tile)
 {
-    const int d = *const_cast<const volatile int *>(dead + seq % kDeadSlots);
-    return __shfl_sync(0xffffffffu, d, 0) == kSlabWarps;
+    const int d = *const_cast<const volatile int *>(done + (threadIdx.x & 31) % kSlabWarps);
+    return __all_sync(0xffffffffu, d == tile);
 }
 
-// A consumer warp's report, once per tile (`slot` is then -1): no lane needs another slab.
-__device__ __forceinline__ void report_dead(int *dead, int &slot, bool need)
+// A consumer warp's report after a stage of `tile`: none of its lanes needs another slab.  Nothing
+// of it stays in a register while the warp marches.
+__device__ __forceinline__ void report_done(int *done, const int &tile, bool need)
 {
-    if (slot >= 0 && !__any_sync(0xffffffffu, need)) {
-        if ((threadIdx.x & 31) == 0) atomicAdd(dead + slot, 1);
-        slot = -1;
-    }
+    if (!__any_sync(0xffffffffu, need) && (threadIdx.x & 31) == 0)
+        *const_cast<volatile int *>(done + (threadIdx.x >> 5)) = tile;
 }
 
 // The producer warp's ring: stage take / publish with every wait bounded.
@@ -467,8 +465,8 @@ struct SlabRing {
             return -1;
         return st;
     }
-    // a stage that carries only its header (a tile's start: and its entry of sh.dead)
-    __device__ __forceinline__ bool post_plain(int type, int tile, int seq = 0)
+    // a stage that carries only its header
+    __device__ __forceinline__ bool post_plain(int type, int tile)
     {
         const int st = take();
         if (st < 0) return false;
@@ -476,8 +474,6 @@ struct SlabRing {
             SlabHdr h{};
             h.type = type;
             h.tile = tile;
-            h.s_lo = seq % kDeadSlots;
-            if (type == kStageTile) sh.dead[seq % kDeadSlots] = 0;
             sh.hdr[st] = h;
             mbar_arrive(&sh.full[st]);
         }
@@ -493,7 +489,7 @@ struct SlabRing {
 // wait gave up.
 template <class EP, int M, bool EARLY>
 __device__ __forceinline__ bool produce_tile(const TileRays &r, bool persp, const CUtensorMap *map_n,
-                                             const CUtensorMap *map_w, const RenderArgs &a, int tile, int seq,
+                                             const CUtensorMap *map_w, const RenderArgs &a, int tile,
                                              unsigned char *stages, SlabRing &ring)
 {
     using G = SlabGeom<EP>;
@@ -511,7 +507,7 @@ __device__ __forceinline__ bool produce_tile(const TileRays &r, bool persp, cons
             hi_c = min(hi_c, e);
     }
     int cur = dir > 0 ? lo_c : hi_c;
-    while (cur >= lo_c && cur <= hi_c && !(EARLY && tile_dead(ring.sh.dead, seq))) {
+    while (cur >= lo_c && cur <= hi_c && !(EARLY && tile_done(ring.sh.done, tile))) {
         const int len = lane + 1;
         const int c0 = dir > 0 ? cur : max(cur - len + 1, lo_c);
         const int c1 = dir > 0 ? min(cur + len - 1, hi_c) : cur;
@@ -566,7 +562,7 @@ __device__ void slab_producer(const CUtensorMap *maps, const shw_camera &cam, co
     const int lane = threadIdx.x & 31;
     SlabRing ring{sh, sa};
     bool ok = true;
-    for (int seq = 0; ok; ++seq) {
+    while (ok) {
         unsigned t = 0;
         if (lane == 0) t = atomicAdd(sa.ctr, 1u);
         t = __shfl_sync(0xffffffffu, t, 0);
@@ -574,18 +570,18 @@ __device__ void slab_producer(const CUtensorMap *maps, const shw_camera &cam, co
             ring.post_plain(kStageExit, 0);
             break;
         }
-        if (!ring.post_plain(kStageTile, (int)t, seq)) break;
+        if (!ring.post_plain(kStageTile, (int)t)) break;
         int tx, ty;
         slab_tile((int)t, a, tx, ty);
         const TileRays r = tile_rays(cam, tx * kSlabTW, ty * kSlabTH);
         const bool persp = !cam.ortho;
         // maps: x-major; y-major narrow, wide; z-major narrow, wide
         if (r.major == 0)
-            ok = produce_tile<EP, 0, EARLY>(r, persp, &maps[0], &maps[0], a, (int)t, seq, stages, ring);
+            ok = produce_tile<EP, 0, EARLY>(r, persp, &maps[0], &maps[0], a, (int)t, stages, ring);
         else if (r.major == 1)
-            ok = produce_tile<EP, 1, EARLY>(r, persp, &maps[1], &maps[2], a, (int)t, seq, stages, ring);
+            ok = produce_tile<EP, 1, EARLY>(r, persp, &maps[1], &maps[2], a, (int)t, stages, ring);
         else
-            ok = produce_tile<EP, 2, EARLY>(r, persp, &maps[3], &maps[4], a, (int)t, seq, stages, ring);
+            ok = produce_tile<EP, 2, EARLY>(r, persp, &maps[3], &maps[4], a, (int)t, stages, ring);
         if (ok) ok = ring.post_plain(kStageTileEnd, (int)t);
     }
     // the CTA may not exit while a tensor copy into its shared memory is in flight: wait
@@ -620,7 +616,6 @@ __device__ void slab_consumer(const S &s, const shw_camera &cam, const RenderArg
     long long X = 0, Y = 0, Z = 0, pix = 0;
     int N = 0, k = 0, kb = 0, done = 0;
     bool has = false, live = false;
-    int slot = -1;  // the tile's entry of sh.dead
     for (int posts = 0;; ++posts) {
         const int si = posts % kSlabStages;
         if (!slab_wait(&sh.full[si], (uint32_t)((posts / kSlabStages) & 1), quit, sa.err, sa.polls)) return;
@@ -637,7 +632,6 @@ __device__ void slab_consumer(const S &s, const shw_camera &cam, const RenderArg
             N = hit ? min(r.N, a.nmax) : 0;
             st = St{};
             done = 0;
-            slot = h.s_lo;
             live = N > 0;
             if (live) {
                 int ka;
@@ -699,7 +693,7 @@ __device__ void slab_consumer(const S &s, const shw_camera &cam, const RenderArg
         }
         __syncwarp();
         if constexpr (is_composite<MODE>)  // (the other modes take every sample)
-            if (h.type != kStageTileEnd) report_dead(sh.dead, slot, live && k < kb);
+            report_done(sh.done, sh.hdr[si].tile, live && k < kb);
         if (lane == 0) mbar_arrive(&sh.empty[si]);
     }
 }
@@ -723,6 +717,7 @@ __global__ void __launch_bounds__(kSlabThreads, kSlabMinBlocks)
             mbar_init(&sh.full[i], 1);
             mbar_init(&sh.empty[i], kSlabWarps);
         }
+        for (int w = 0; w < kSlabWarps; ++w) sh.done[w] = -1;
         sh.quit = 0;
         fence_barrier_init();
     }
