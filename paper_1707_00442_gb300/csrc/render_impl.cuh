@@ -15,6 +15,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 #include <type_traits>
 
 #include "common.cuh"
@@ -894,22 +895,35 @@ int sm_count();
 // from a global counter until none is left, so no SM idles while rays of very
 // different lengths finish and no CTA launch overhead is paid per tile.
 //
-// Resident CTAs per SM the kernel is compiled for (1: what the compiler takes, 8 for most, from
-// the registers of the ray set-up).  It waits on its gathers, so where the march itself needs
-// few registers more warps in flight win: nearest sampling of 512^3 on 1000 x 1000 861 us with
-// 11, 709 with 12 (80 registers; 16: 740), compositing 750 x 750 x 70 448 / 336 / 345 with
-// 8 / 12 / 16, the ratio of two cubes, which holds 32 corners, 240 / 206 / 213 / 373 with
-// 8 / 10 / 12 / 16 (spills).  The other trilinear modes gain nothing and lose where neighbouring
-// rays share their loads (395 x 395 x 41 along z: 172 us with 8, 208 with 12).
+// Each kernel is compiled in the form that the compiler takes (8 to 11 resident CTAs per SM, from
+// the registers of the ray set-up) and, where the march itself needs few registers, in one for
+// more: it waits on its gathers, so with enough rays more warps in flight win.  Nearest sampling
+// of 512^3 on 1000 x 1000 861 us with 11, 709 with 12 (80 registers; 16: 740), compositing
+// 750 x 750 x 70 448 / 336 / 345 with 8 / 12 / 16, the ratio of two cubes, which holds 32 corners,
+// 240 / 206 / 213 / 373 with 8 / 10 / 12 / 16 (spills).  The other trilinear modes gain nothing and
+// lose where neighbouring rays share their loads (395 x 395 x 41 along z: 172 us with 8, 208 with 12).
 template <int MODE, int INTERP, int SMK>
 constexpr int render_min_ctas()
 {
     if (SMK > 0) return 1;
-    if (INTERP == SHW_NEAREST || is_composite<MODE>) return 12;
-    return two_cubes<MODE> ? 10 : 1;
+    if (two_cubes<MODE>) return INTERP == SHW_NEAREST ? 1 : 10;
+    return INTERP == SHW_NEAREST || is_composite<MODE> ? 12 : 1;
 }
-template <int MODE, int INTERP, class S, int SMK = 0>
-__global__ void __launch_bounds__(kRenderThreads, (render_min_ctas<MODE, INTERP, SMK>()))
+// The form for more CTAs serves views of at least kManyWarps warps' pixels (below, fewer
+// registers only slow each ray: over 254 ratios of two cubes 0.72 to 1.41 of the other form's time
+// below and 0.79 to 1.00 above; 347 nearest and 344 compositing renders 0.70 to 1.41 below, 0.73 to
+// 1.01 above), and cubes that the second-level cache still helps with: above these sizes more rays
+// in flight draw their planes from HBM over and over (the ratio of two 641^3 cubes on 1000 x 1000
+// at yaw 70 4.87 ms, 5.56 with 10 per SM; compositing 1024^3 clipped at yaw 60 6.6 and 14.1).
+constexpr double kManyWarps = 10000.0;
+template <int MODE, int INTERP>
+constexpr double render_max_voxels()
+{
+    if (INTERP == SHW_NEAREST) return 1e30;
+    return two_cubes<MODE> ? 67108864.0 : 536870912.0;
+}
+template <int MODE, int INTERP, class S, int SMK = 0, int MINB = render_min_ctas<MODE, INTERP, SMK>()>
+__global__ void __launch_bounds__(kRenderThreads, MINB)
     render_kernel_persistent(S s, S s2, shw_camera cam, RenderArgs a, unsigned *ctr, int nwarp_tiles)
 {
     const int lane = threadIdx.x & 31;
@@ -966,6 +980,29 @@ inline void project_centre(const shw_camera &c, int nx, int ny, int nz, float &p
     py = 0.5f * (1.0f - ys) * c.height;
 }
 
+// Voxels per pixel at the cube's centre.
+inline double centre_pitch(const shw_camera &c, int nx, int ny, int nz)
+{
+    if (c.ortho) return 2.0 * c.ortho_half_h / c.height;
+    const double n[3] = {(double)nx, (double)ny, (double)nz};
+    double len2 = 0.0, depth = 0.0;
+    for (int k = 0; k < 3; ++k) {
+        len2 += (double)c.fwd[k] * c.fwd[k];
+        depth += (0.5 * (n[k] - 1.0) - c.eye[k]) * c.fwd[k];
+    }
+    return 2.0 * c.tan_half_fovy * std::fabs(depth) / len2 / c.height;
+}
+
+// About how many pixels see the cube: its parallel projection at its centre's scale.
+inline double covered_pixels(const shw_camera &c, int nx, int ny, int nz)
+{
+    const double len = std::sqrt((double)c.fwd[0] * c.fwd[0] + (double)c.fwd[1] * c.fwd[1] + (double)c.fwd[2] * c.fwd[2]);
+    const double area = ((double)ny * nz * std::fabs(c.fwd[0]) + (double)nx * nz * std::fabs(c.fwd[1]) +
+                         (double)nx * ny * std::fabs(c.fwd[2])) / len;  // voxels^2
+    const double pitch = centre_pitch(c, nx, ny, nz), all = (double)c.width * c.height;
+    return area < all * pitch * pitch ? area / (pitch * pitch) : all;
+}
+
 // Host-side launch for one storage type (instantiated per storage in its own TU).
 // SMK > 0: the in-ray smoothing instances (persistent form only; see render_pixel).
 template <int SMK, class S>
@@ -987,30 +1024,30 @@ shw_status launch_render_modes(int mode, int interp, const S &s, const S &s2, co
     unsigned *ctr = SHW_RENDER_PERSISTENT ? work_counter(st) : nullptr;
     const int nsm = sm_count();
     const int nwarp_tiles = (int)(tiles * kCtaWarps);
-    // persistent grid: as many CTAs as fit on the device at once (at most one per tile).  An
-    // image of only a few tiles per CTA takes fewer of the raised counts, down to 8 per SM: more would leave
-    // nothing to even out the long rays with (128^3 on 500 x 500, compositing: 137 us with 8 per
-    // SM, 193 with 12; 1000 x 1000: 389 and 383).  Nearest sampling's rays are too short to
-    // mind (45 us with 11 per SM, 53 with 8).  Compositing a cube of more than 2^29 voxels also
-    // stays at 8: more rays in flight than that draw their planes from HBM over and over (1024^3 on
-    // 1000 x 1000, clipped, gathered: 14.1 ms with 12 per SM, 6.6 with 8 at yaw 60, though 3.1 and
-    // 4.3 along z; 641^3: 3.1 and 2.7, 1.9 and 2.4).
+    // persistent grid: as many CTAs as fit on the device at once (at most one per tile); of the
+    // raised counts no more than leave four tiles to each, to even out the long rays with (128^3 on
+    // 500 x 500, compositing: 137 us with 8 per SM, 193 with 12; 1000 x 1000: 389 and 383).  Nearest
+    // sampling's rays are too short to mind.
     auto persistent = [&](auto kern, int per_sm, bool more_ctas) {
         long long g = std::min<long long>((long long)per_sm * nsm, tiles);
-        if (SMK == 0 && interp != SHW_NEAREST && more_ctas) g = std::min(g, std::max(tiles / 4, 8LL * nsm));
-        if (SMK == 0 && interp != SHW_NEAREST && more_ctas && (double)s.nx * s.ny * s.nz > 536870912.0)
-            g = std::min(g, 8LL * nsm);
+        if (more_ctas && interp != SHW_NEAREST) g = std::min(g, std::max(tiles / 4, 8LL * nsm));
         kern<<<(unsigned)std::max<long long>(g, 1), block, 0, st>>>(s, s2, cam, a, ctr, nwarp_tiles);
     };
+    const bool many = covered_pixels(cam, s.nx, s.ny, s.nz) >= 32.0 * kManyWarps;
+    const double vox = (double)s.nx * s.ny * s.nz;
     if (SMK > 0 && (ctr == nullptr || nsm <= 0)) return SHW_ECUDA;
 #define SHW_LAUNCH(M, I)                                                       \
     do {                                                                       \
         if constexpr (SMK > 0)                                                 \
             persistent(render_kernel_persistent<M, I, S, SMK>,                 \
                        resident_per_sm<render_kernel_persistent<M, I, S, SMK>>(), false); \
-        else if (ctr != nullptr && nsm > 0)                                    \
+        else if (ctr != nullptr && nsm > 0 && render_min_ctas<M, I, 0>() > 1 && many && \
+                 vox <= render_max_voxels<M, I>())                             \
             persistent(render_kernel_persistent<M, I, S>,                      \
-                       resident_per_sm<render_kernel_persistent<M, I, S>>(), render_min_ctas<M, I, 0>() > 8); \
+                       resident_per_sm<render_kernel_persistent<M, I, S>>(), true); \
+        else if (ctr != nullptr && nsm > 0)                                    \
+            persistent(render_kernel_persistent<M, I, S, 0, 1>,                \
+                       resident_per_sm<render_kernel_persistent<M, I, S, 0, 1>>(), false); \
         else                                                                   \
             render_kernel<M, I, S><<<grid, block, 0, st>>>(s, s2, cam, a);     \
     } while (0)

@@ -1,0 +1,26 @@
+// dispatch_rules.cu -- host program of test_dispatch_rules_host.py: reads requests (a rule's name, the
+// camera, the cube's dims and a number) and prints 1 or 0 for each, the rule's choice.
+#include <cstdio>
+#include <cstring>
+
+#include "render_impl.cuh"
+
+using namespace shw;
+
+int main()
+{
+    char rule[32];
+    shw_camera c{};
+    int n[3], k;
+    auto three = [](float *v) { return std::scanf("%f %f %f", v, v + 1, v + 2) == 3; };
+    while (std::scanf("%31s", rule) == 1) {
+        if (!three(c.eye) || !three(c.right) || !three(c.up) || !three(c.fwd) ||
+            std::scanf("%f %f %d %d %d %d %d %d %d", &c.tan_half_fovy, &c.ortho_half_h, &c.ortho, &c.width, &c.height, n,
+                       n + 1, n + 2, &k) != 9)
+            return 2;
+        bool yes = false;
+        if (!std::strcmp(rule, "many")) yes = covered_pixels(c, n[0], n[1], n[2]) >= 32.0 * kManyWarps;
+        std::printf("%d\n", yes ? 1 : 0);
+    }
+    return 0;
+}

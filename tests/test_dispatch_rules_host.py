@@ -1,0 +1,36 @@
+"""Where each staged or widened form is taken, on the host (no GPU): the rules are plain host code, compiled
+here and asked about requests whose two routes were measured.  Every time is microseconds on a
+GB300, of the route named first and of the other; the rule must take the faster."""
+import os
+import subprocess
+
+import pytest
+
+import scene
+
+
+@pytest.fixture(scope="module")
+def ask(tmp_path_factory):
+    from paper_1707_00442_gb300 import build
+    src = os.path.join(os.path.dirname(__file__), "dispatch_rules.cu")
+    exe = str(tmp_path_factory.mktemp("rules") / "dispatch_rules")
+    subprocess.run([build.nvcc(), *build._flags(), src, "-o", exe], check=True)
+
+    def run(rule, dims, cam, k=0):
+        v = [*cam.eye, *cam.right, *cam.up, *cam.fwd, cam.tan_half_fovy, cam.ortho_half_h]
+        line = " ".join([rule, *(repr(float(x)) for x in v),
+                         *(str(int(x)) for x in (cam.ortho, cam.width, cam.height, *dims, k))])
+        r = subprocess.run([exe], input=line, capture_output=True, text=True, timeout=60)
+        assert r.returncode == 0, r.stderr
+        return int(r.stdout)
+    return run
+
+
+@pytest.mark.parametrize("dims,yaw,W,H,more,plain", [
+    ((50, 50, 37), 70, 1000, 1000, 204, 240), ((750, 750, 70), 20, 1000, 1000, 333, 446),
+    ((301, 300, 300), 30, 1600, 1600, 2583, 2871),
+    ((65, 66, 67), 30, 64, 64, 75, 58), ((201, 200, 200), 0, 200, 200, 210, 165),
+    ((68, 388, 169), 227, 169, 549, 433, 321), ((419, 52, 107), 172, 132, 753, 113, 81)])
+def test_more_resident_ctas(ask, dims, yaw, W, H, more, plain):
+    """Gathered ratios of two cubes, the second compositing: compiled for more resident CTAs, and not."""
+    assert ask("many", dims, scene.orbit_camera(dims, yaw, 20, W, H)) == (more < plain)
