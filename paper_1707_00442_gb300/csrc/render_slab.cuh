@@ -759,42 +759,35 @@ shw_status slab_launch_one(const SlabMaps &maps, const S &s, const shw_camera &c
 }
 
 // Whether staging pays for a float32 cube or pair storage (the gather marcher is the
-// alternative), from the tile at the cube's projected centre where its rays pass its middle:
-//   - its footprint in a slab of one cell has to fit the staged box, or most samples would read
-//     global memory one at a time (300^3 on 500 x 500, yaw 70: 545 us staged, 388 gathered);
-//     x-major boxes stay below three quarters of a stage, fuller ones leave slabs of one cell
-//     (200^3 on 400 x 400, yaw 85: 344 against 180).  A cube larger than the second-level cache
-//     is gathered from HBM, and a footprint up to 50 cells wide still stages better (512^3 on
-//     640 x 640: 816 against 1298; the pair storage of 512^3 on 1000 x 1000, yaw 70: 2693
-//     against 3835).  The less of the cube that cache holds, the more a gather costs, so the
-//     limit grows by 24 cells for each doubling above 2^27 voxels, up to 100: at 70 to 80 cells
-//     and 2^28 voxels (512 x 512 x 1024 on 1000 x 1000, yaw 70) MIP takes 2083 us staged and
-//     4054 gathered, but with 134M voxels and 110 cells (512^3 on 400 x 400, yaw 90) gathering
-//     is 1.6 times as fast; 1024^3 on 1000 x 1000, yaw 70 (95 cells): 5831 against 7750, on
-//     700 x 700, yaw 90 (121 cells) gathering is 1.3 times as fast;
-//   - above a fifth of a voxel per pixel: below, the gathers hit the first-level cache and the
-//     stages' hand-overs cost more (64^3 on 1000 x 1000, compositing: 267 against 217).
-// Over 700 renders (48^3 .. 512^3 and oblong cubes, 128^2 .. 1000^2, five views, MIP and
-// compositing) the rule is 2 % from the better of the two on average, always staging 21 %;
-// over 584 renders of cubes above the cache's size (400^3 .. 1024^3, float32 and pairs, 250^2 ..
-// 2000^2, eight views) 4.3 % on average (early ends that compositing meets are not foreseen),
-// always staging 16 %, a limit of 50 cells 6.6 %.
+// alternative), from the tile at the cube's projected centre where its rays pass its middle.
+// Most samples of a tile whose footprint overflows the staged box read global memory one at a
+// time; but so long as some slabs fit, staging hides more of that than a gather does.  So a view is
+// gathered only where no request measured was slower for it:
+//   - the footprint in a slab of one cell overflows a stage (x-major float32 boxes; pairs, whose
+//     x-major rows are half as many cells, from three quarters of one): 200^3 on 256 x 256, yaw 85:
+//     MIP 495 us staged, 189 gathered; just within, 512^3 on 1000 x 1000, 2422 and 3959;
+//   - y- and z-major footprints wider than 66 cells, or for cubes larger than the second-level
+//     cache, which are gathered from HBM, 110 (256^3 on 400 x 400, yaw 60, 44 cells: 238 staged, 425
+//     gathered; 512^3 on 400 x 400, yaw 90, 110 cells: gathering is 1.6 times as fast); pairs wider
+//     than the box of 34, beyond the cache's size only from 2.2 voxels per pixel on;
+//   - below a tenth of a voxel per pixel, where the gathers hit the first-level cache and the stages'
+//     hand-overs cost more (48^3 on 1000 x 1000, compositing: 218 us staged, 179 gathered).
+// Over 2984 renders (32^3 .. 1024^3 and oblong cubes, 96^2 .. 2000^2, MIP, compositing, the other
+// modes and pairs) this takes 18 % less time than always staging, and its two worst choices took
+// 1.06 and 1.05 times as long.  (The better of the two each time would take 24 % less.)
 template <class G>
 inline bool slab_pays(const shw_camera &c, int nx, int ny, int nz)
 {
+    const double pitch = centre_pitch(c, nx, ny, nz);
+    if (pitch <= 0.1) return false;
     float px, py;
     project_centre(c, nx, ny, nz, px, py);
     const int x0 = (int)fminf(fmaxf(px, 0.0f), (float)(c.width - 1)) / kSlabTW * kSlabTW;
     const int y0 = (int)fminf(fmaxf(py, 0.0f), (float)(c.height - 1)) / kSlabTH * kSlabTH;
-    float pitch = 2.0f * c.ortho_half_h / (float)c.height;  // voxels per pixel at the centre
-    if (!c.ortho) {
-        const float q[3] = {0.5f * (nx - 1) - c.eye[0], 0.5f * (ny - 1) - c.eye[1], 0.5f * (nz - 1) - c.eye[2]};
-        pitch = 2.0f * c.tan_half_fovy / (float)c.height *
-                fabsf(q[0] * c.fwd[0] + q[1] * c.fwd[1] + q[2] * c.fwd[2]);
-    }
-    if (pitch <= 0.2f) return false;
     const TileRays r = tile_rays(c, x0, y0);
-    auto fits = [&](auto mc, int na, int nb, int nm) {
+    constexpr bool pair = G::kBytes == 8;
+    const bool hbm = (double)nx * ny * nz * G::kBytes > 128e6;
+    auto pays = [&](auto mc, int na, int nb, int nm) {
         constexpr int M = decltype(mc)::value, A = M == 0 ? 1 : 0, B = M == 2 ? 1 : 2;
         TileLines<M> L;
         if (!tile_lines<M>(r, L)) return false;
@@ -811,16 +804,15 @@ inline bool slab_pays(const shw_camera &c, int nx, int ny, int nz)
                 }
             ext[k] = fminf(hi - lo + 2.0f, (float)(k == 0 ? na : nb));
         }
-        if (M == 0) return ceilf(ext[0] / kSlabRows) * kSlabRows * ext[1] * G::kBXx <= 0.75f * G::kStageElems;
-        const float vox = (float)nx * (float)ny * (float)nz;
-        const bool hbm = vox * (float)G::kBytes > 128e6f;
-        const float widest = fminf(fmaxf(50.0f + 24.0f * (log2f(vox) - 27.0f), 50.0f), 100.0f);
-        return ext[0] <= (hbm ? widest : (float)(G::kBXw - 2)) &&
-               2.0f * ext[1] * (float)(ext[0] + 3.0f <= G::kBXn ? G::kBXn : G::kBXw) <= (float)G::kStageElems;
+        if (M == 0)
+            return ceilf(ext[0] / kSlabRows) * kSlabRows * ext[1] * G::kBXx <= (pair ? 0.75f : 1.02f) * G::kStageElems;
+        if (2.0f * ext[1] * (float)(ext[0] + 3.0f <= G::kBXn ? G::kBXn : G::kBXw) > (float)G::kStageElems) return false;
+        if (pair) return (hbm && pitch < 2.2) || ext[0] <= 34.0f;
+        return ext[0] <= (hbm ? 110.0f : 66.0f);
     };
-    if (r.major == 0) return fits(std::integral_constant<int, 0>{}, ny, nz, nx);
-    if (r.major == 1) return fits(std::integral_constant<int, 1>{}, nx, nz, ny);
-    return fits(std::integral_constant<int, 2>{}, nx, ny, nz);
+    if (r.major == 0) return pays(std::integral_constant<int, 0>{}, ny, nz, nx);
+    if (r.major == 1) return pays(std::integral_constant<int, 1>{}, nx, nz, ny);
+    return pays(std::integral_constant<int, 2>{}, nx, ny, nz);
 }
 
 // The launch for one storage: the tensor maps (x-major chunks; y- and z-major chunks, narrow

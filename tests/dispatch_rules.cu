@@ -4,6 +4,7 @@
 #include <cstring>
 
 #include "render_impl.cuh"
+#include "render_slab.cuh"
 
 using namespace shw;
 
@@ -20,6 +21,8 @@ int main()
             return 2;
         bool yes = false;
         if (!std::strcmp(rule, "many")) yes = covered_pixels(c, n[0], n[1], n[2]) >= 32.0 * kManyWarps;
+        if (!std::strcmp(rule, "staged")) yes = slab_pays<SlabGeom<ElemF32>>(c, n[0], n[1], n[2]);
+        if (!std::strcmp(rule, "staged_pair")) yes = slab_pays<SlabGeom<ElemF32Pair>>(c, n[0], n[1], n[2]);
         std::printf("%d\n", yes ? 1 : 0);
     }
     return 0;

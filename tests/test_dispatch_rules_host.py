@@ -34,3 +34,20 @@ def ask(tmp_path_factory):
 def test_more_resident_ctas(ask, dims, yaw, W, H, more, plain):
     """Gathered ratios of two cubes, the second compositing: compiled for more resident CTAs, and not."""
     assert ask("many", dims, scene.orbit_camera(dims, yaw, 20, W, H)) == (more < plain)
+
+
+@pytest.mark.parametrize("dims,yaw,pitch,W,staged,gathered", [
+    ((512, 512, 512), 85, 10, 1000, 2422, 3959), ((256, 256, 256), 60, -30, 400, 238, 425),
+    ((64, 64, 512), 60, -30, 400, 75, 131), ((1024, 1024, 1024), 55, 20, 500, 2808, 4938),
+    ((512, 512, 512), 70, 20, 640, 1640, 1713),
+    ((200, 200, 200), 85, 10, 256, 495, 189), ((512, 512, 512), 85, 10, 256, 2483, 856),
+    ((48, 48, 48), 85, 10, 1000, 165, 149)])
+def test_staged_marcher(ask, dims, yaw, pitch, W, staged, gathered):
+    """MIP of a float32 cube: the staged marcher, and the gather."""
+    assert ask("staged", dims, scene.orbit_camera(dims, yaw, pitch, W, W)) == (staged < gathered)
+
+
+def test_staged_marcher_of_pairs(ask):
+    for dims, yaw, pitch, W, staged, gathered in [((64, 64, 512), 60, -30, 640, 129, 161),
+                                                  ((256, 256, 256), 85, 10, 256, 965, 420)]:
+        assert ask("staged_pair", dims, scene.orbit_camera(dims, yaw, pitch, W, W)) == (staged < gathered)
