@@ -36,12 +36,10 @@ shw_status render_axis(int mode, int interp, const shw_volume &v, const shw_came
     const double ext_x = (kAxTX - 1) * std::fabs(ax) + (kAxTY - 1) * std::fabs(bx);
     const double ext_y = (kAxTX - 1) * std::fabs(ay) + (kAxTY - 1) * std::fabs(by);
     AxisArgs A{};
-    // rows that no tensor copy takes: row copies, with 32-bit element indexes.  A few planes under
-    // a small image are gathered as fast (71 x 71 x 48 on 71^2: 48 us gathered, 52 by row copies;
-    // 67 x 67 x 193 on 134^2: 137 and 121, 601 x 601 x 300 on 601^2: 961 and 494)
+    // rows that no tensor copy takes: row copies, with 32-bit element indexes
     A.rows = v.nx % 4 != 0 || !aligned(v.data, 16);
     if (A.rows && ((long long)v.nx * v.ny * v.nz >= (1ll << 31) ||
-                   (v.nz < 96 && (long long)c.width * c.height < 65536 && !debug(SHW_DEBUG_REQUIRE_STAGING))))
+                   (!axis_rows_pay(mode, interp, c, v.nz) && !debug(SHW_DEBUG_REQUIRE_STAGING))))
         return SHW_EUNSUPPORTED;
     A.goff = (int)((reinterpret_cast<uintptr_t>(v.data) >> 2) & 3);
     const int kmode = (mode == SHW_MIP && a.index == nullptr) ? kMipValue : mode;

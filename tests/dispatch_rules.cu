@@ -3,6 +3,7 @@
 #include <cstdio>
 #include <cstring>
 
+#include "render_axis.cuh"
 #include "render_impl.cuh"
 #include "render_slab.cuh"
 
@@ -23,6 +24,8 @@ int main()
         if (!std::strcmp(rule, "many")) yes = covered_pixels(c, n[0], n[1], n[2]) >= 32.0 * kManyWarps;
         if (!std::strcmp(rule, "staged")) yes = slab_pays<SlabGeom<ElemF32>>(c, n[0], n[1], n[2]);
         if (!std::strcmp(rule, "staged_pair")) yes = slab_pays<SlabGeom<ElemF32Pair>>(c, n[0], n[1], n[2]);
+        if (!std::strcmp(rule, "rows")) yes = axis_rows_pay(k, SHW_TRILINEAR, c, n[2]);
+        if (!std::strcmp(rule, "rows_nearest")) yes = axis_rows_pay(k, SHW_NEAREST, c, n[2]);
         std::printf("%d\n", yes ? 1 : 0);
     }
     return 0;

@@ -7,6 +7,7 @@ import subprocess
 import pytest
 
 import scene
+from scene.camera import ortho_axis_camera
 
 
 @pytest.fixture(scope="module")
@@ -51,3 +52,16 @@ def test_staged_marcher_of_pairs(ask):
     for dims, yaw, pitch, W, staged, gathered in [((64, 64, 512), 60, -30, 640, 129, 161),
                                                   ((256, 256, 256), 85, 10, 256, 965, 420)]:
         assert ask("staged_pair", dims, scene.orbit_camera(dims, yaw, pitch, W, W)) == (staged < gathered)
+
+
+MIP, COMPOSITE, MOMENT1 = 0, 2, 5
+
+
+@pytest.mark.parametrize("rule,n,nz,mode,rows,gathered", [
+    ("rows", 350, 454, MIP, 296, 749), ("rows", 601, 300, MIP, 459, 958), ("rows", 601, 300, COMPOSITE, 636, 789),
+    ("rows", 71, 300, COMPOSITE, 213, 151), ("rows", 65, 97, MOMENT1, 98, 72), ("rows", 131, 400, MOMENT1, 340, 275),
+    ("rows_nearest", 601, 300, MIP, 440, 595), ("rows_nearest", 65, 97, MIP, 80, 54),
+    ("rows_nearest", 131, 400, MIP, 271, 187), ("rows_nearest", 401, 20, COMPOSITE, 74, 52)])
+def test_sweep_by_row_copies(ask, rule, n, nz, mode, rows, gathered):
+    """Spectral-axis views of n x n x nz cubes, one pixel a voxel: the sweep by row copies, and the gather."""
+    assert ask(rule, (n, n, nz), ortho_axis_camera((n, n, nz), n, n), mode) == (rows < gathered)
