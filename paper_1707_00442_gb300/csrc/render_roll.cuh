@@ -896,20 +896,44 @@ shw_status roll_launch_one(const RollMaps &maps, const S &s, const shw_camera &c
     return after_launch();
 }
 
-// Whether the ring pays (else the samples are gathered): its hand-overs and halo planes are a
-// fixed cost per tile, and the gathers of a small cube hit the caches.  Over 864 renders (32^3 ..
-// 320^3 and oblong cubes, 128^2 .. 1000 x 800, three views) the rule is 2 to 4 % from the better of
-// the two marchers; for 9 taps always gathering is 24 % off and never 12 %, for the box 5 % and
-// 42 %.  Below 64 voxels on an axis most samples' taps clamp; few taps (1 pair) and row copies
-// need a larger cube, and the box, two fetches a sample when gathered, needs 10^7 voxels and
-// tensor copies (512^3 on 1000 x 1000: 9 taps 53.9 ms gathered, 11.5 staged; the 5-box 5.86 and
-// 2.32).
+// Whether the ring pays (else the samples are gathered).  Its hand-overs and halo planes are a fixed
+// cost per tile and it keeps one CTA per tile, so it needs tiles that fill the device and
+// footprints that are not much wider than the taps' reach; a gather costs least where a warp's rays
+// share rows of the cube (y- and z-major views), most in x-major ones and where the cube exceeds the
+// second-level cache (from 3 x 10^7 voxels on).  Compositing's gathers stop with the ray, the ring
+// with the tile.  From the major axis of the tile at the cube's projected centre, the voxels per
+// pixel there and the tiles that see the cube.  Over 2766 renders (32^3 .. 640^3 and oblong cubes,
+// 96^2 .. 1000^2, eleven views and random ones, 3 to 13 taps, boxes of 3 to 9) the ring took 0.10 to
+// 1.04 of the gather's time where this takes it, up to 11 times as long elsewhere (9 taps, 512^3 on
+// 1000 x 1000: MIP at yaw 30 24.1 ms gathered, 8.7 staged, at yaw 100 82.6 and 7.9, looking down
+// at yaw 20 13.0 and 8.5, compositing 7.1 and 7.4; 129^3 on 128 x 128, MIP along z 0.33 and 0.59).
 template <int KIND>
-inline bool roll_pays(const int n[3], bool tmaps, int ntaps)
+inline bool roll_pays(const shw_camera &cam, const int n[3], bool tmaps, int ntaps, bool composite, float xbias)
 {
-    const double vox = (double)n[0] * n[1] * n[2];
-    if (KIND == kRollBox) return tmaps && vox >= 1e7;
-    return std::min(n[0], std::min(n[1], n[2])) >= 64 && ((tmaps && ntaps >= 2) || vox >= 2e6);
+    const double vox = (double)n[0] * n[1] * n[2], pitch = centre_pitch(cam, n[0], n[1], n[2]);
+    const double tiles = covered_pixels(cam, n[0], n[1], n[2]) / (kSlabTW * kSlabTH);
+    const int least = std::min(n[0], std::min(n[1], n[2]));
+    float px, py;
+    project_centre(cam, n[0], n[1], n[2], px, py);
+    const int on[3] = {1, 1, 1};
+    const int major = roll_rays(cam, (int)fminf(fmaxf(px, 0.0f), (float)(cam.width - 1)) / kSlabTW * kSlabTW,
+                                (int)fminf(fmaxf(py, 0.0f), (float)(cam.height - 1)) / kSlabTH * kSlabTH, on, xbias)
+                          .major;
+    const bool big = vox >= 3e7;
+    if (KIND == kRollBox) {  // two fetches a sample when gathered: large cubes by tensor copies only
+        if (!tmaps || vox < 1e7) return false;
+        if (composite) return big && pitch <= 1.25 && (major == 0 || (major == 2 && tiles >= 450.0));
+        if (big) return pitch <= 1.6;
+        return least >= 100 && (major == 0 ? pitch <= 0.9 : tiles >= 450.0 && pitch <= 0.7);
+    }
+    // few taps and row copies need a larger cube; below 64 voxels on an axis most taps clamp
+    if (least < 64 || !((tmaps && ntaps >= 2) || vox >= 2e6)) return false;
+    if (composite) {
+        if (!big) return major == 0 && vox >= 3e6 && least >= 100 && pitch <= 0.9;
+        return major == 0 ? pitch <= 1.25 : major == 2 && tiles >= 450.0 && pitch <= 2.5;
+    }
+    if (big) return pitch <= 2.5 && tiles >= (major == 2 ? 450.0 : 300.0);
+    return major == 0 ? vox >= 2e6 && tiles >= 152.0 && pitch <= 0.9 : tiles >= 608.0 && pitch <= 0.6;
 }
 
 // In-ray smoothing of a float32 cube through the rolling marcher; SHW_EUNSUPPORTED when it
@@ -929,7 +953,13 @@ shw_status roll_launch(int mode, const shw_volume &v, const shw_camera &cam, con
             ra.halo = std::max(ra.halo, (int)((o + 0xffffffffLL) >> 32));
         }
     const bool tmaps = v.nx % 4 == 0 && aligned(v.data, 16);
-    if (!debug(SHW_DEBUG_REQUIRE_STAGING) && !roll_pays<KIND>(n, tmaps, a0.smooth_n)) return SHW_EUNSUPPORTED;
+    // Taps: the true major axis (the planes hold the taps' reach on both sides, and only small
+    // slopes keep two CTAs on an SM).  The box: x-major planes cost the producer a transposition,
+    // so steep y- and z-major ones are taken up to a slope of 3.
+    ra.xbias = KIND == kRollTaps ? 1.0f : 3.0f;
+    const bool composite = mode == SHW_COMPOSITE || mode == SHW_COMPOSITE_SPECTRAL || mode == SHW_COMPOSITE_RGB;
+    if (!debug(SHW_DEBUG_REQUIRE_STAGING) && !roll_pays<KIND>(cam, n, tmaps, a0.smooth_n, composite, ra.xbias))
+        return SHW_EUNSUPPORTED;
     ra.rows = !tmaps;
     ra.goff = (int)((reinterpret_cast<uintptr_t>(v.data) >> 2) & 3);
     size_t extra = sizeof(RollShared);
@@ -939,10 +969,6 @@ shw_status roll_launch(int mode, const shw_volume &v, const shw_camera &cam, con
         ra.box_mask = len - 1;
         extra += (size_t)len * 32 * kSlabWarps * 4;
     }
-    // Taps: the true major axis (the planes hold the taps' reach on both sides, and only small
-    // slopes keep two CTAs on an SM).  The box: x-major planes cost the producer a transposition,
-    // so steep y- and z-major ones are taken up to a slope of 3.
-    ra.xbias = KIND == kRollTaps ? 1.0f : 3.0f;
     // two CTAs per SM where a step of at least two cells fits, else one
     const int smax = KIND == kRollTaps ? 4 : 12;
     if (!roll_geometry(cam, n, ra.halo, tmaps, kRollBudget2 - (int)extra, smax, 2, ra) &&

@@ -5,6 +5,7 @@
 
 #include "render_axis.cuh"
 #include "render_impl.cuh"
+#include "render_roll.cuh"
 #include "render_slab.cuh"
 
 using namespace shw;
@@ -26,6 +27,11 @@ int main()
         if (!std::strcmp(rule, "staged_pair")) yes = slab_pays<SlabGeom<ElemF32Pair>>(c, n[0], n[1], n[2]);
         if (!std::strcmp(rule, "rows")) yes = axis_rows_pay(k, SHW_TRILINEAR, c, n[2]);
         if (!std::strcmp(rule, "rows_nearest")) yes = axis_rows_pay(k, SHW_NEAREST, c, n[2]);
+        const bool tmaps = n[0] % 4 == 0;
+        if (!std::strcmp(rule, "taps")) yes = roll_pays<kRollTaps>(c, n, tmaps, k, false, 1.0f);
+        if (!std::strcmp(rule, "taps_composite")) yes = roll_pays<kRollTaps>(c, n, tmaps, k, true, 1.0f);
+        if (!std::strcmp(rule, "box")) yes = roll_pays<kRollBox>(c, n, tmaps, k, false, 3.0f);
+        if (!std::strcmp(rule, "box_composite")) yes = roll_pays<kRollBox>(c, n, tmaps, k, true, 3.0f);
         std::printf("%d\n", yes ? 1 : 0);
     }
     return 0;

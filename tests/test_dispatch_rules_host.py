@@ -65,3 +65,16 @@ MIP, COMPOSITE, MOMENT1 = 0, 2, 5
 def test_sweep_by_row_copies(ask, rule, n, nz, mode, rows, gathered):
     """Spectral-axis views of n x n x nz cubes, one pixel a voxel: the sweep by row copies, and the gather."""
     assert ask(rule, (n, n, nz), ortho_axis_camera((n, n, nz), n, n), mode) == (rows < gathered)
+
+
+@pytest.mark.parametrize("rule,dims,yaw,pitch,W,ring,gathered", [
+    ("taps", (512, 512, 512), 100, 10, 1000, 7873, 82899), ("taps", (512, 512, 512), 30, 20, 1000, 8656, 24064),
+    ("taps", (160, 160, 160), 100, 10, 500, 941, 3855), ("taps_composite", (512, 512, 512), 30, 20, 1000, 6667, 16482),
+    ("taps_composite", (512, 512, 512), 20, 75, 1000, 7446, 7167), ("taps", (129, 129, 129), 15, 20, 128, 802, 483),
+    ("taps_composite", (68, 512, 68), 20, 75, 128, 2751, 685), ("taps_composite", (64, 64, 512), 15, 20, 128, 2466, 722),
+    ("box", (512, 512, 512), 100, 10, 1000, 2356, 8305), ("box_composite", (512, 512, 512), 100, 10, 1000, 1820, 4474),
+    ("box", (400, 70, 400), 60, -30, 500, 705, 267), ("box_composite", (320, 320, 320), 15, 20, 128, 718, 264),
+    ("box_composite", (512, 512, 512), 20, 75, 1000, 2265, 2163)])
+def test_rolling_marcher(ask, rule, dims, yaw, pitch, W, ring, gathered):
+    """9 taps, or the box of 3 to 9: the ring, and the gather."""
+    assert ask(rule, dims, scene.orbit_camera(dims, yaw, pitch, W, W), 2) == (ring < gathered)
