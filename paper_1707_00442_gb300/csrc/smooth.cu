@@ -97,14 +97,15 @@ __global__ void __launch_bounds__(32 * (32 / YB)) smooth_kernel(const float *__r
 }
 
 // ---------------------------------------------------------------------------
-// TMA pipeline (radius 1..8, nx a multiple of 4, 16-byte aligned cube).
+// The pipeline (radius 1..8), in two forms: by tensor copies (nx a multiple of 4, a 16-byte
+// aligned cube and outputs aligned for its stores), and by row copies (ROWS: any other cube).
 //
-// Per CTA: a 32 x 32 (x, y) output block and a chunk of z planes.  One thread
-// issues cp.async.bulk.tensor loads of the 52 x (32+2r) input box of each plane
-// into a 3-stage shared ring, signalled through mbarriers; the box's x start
-// (x0 - 8) keeps the TMA coordinate 16-byte aligned.  Out-of-range elements arrive
-// as zeros and, in blocks touching the cube's faces, are replaced by the edge values
-// (clamp-to-edge).  Then:
+// Per CTA: a 32 x 32 (x, y) output block and a chunk of z planes.  The 52 x (32+2r) input box of
+// each plane goes into a 3-stage shared ring, signalled through mbarriers: one thread issues
+// cp.async.bulk.tensor loads, the box's x start (x0 - 8) keeping the TMA coordinate 16-byte
+// aligned, or every thread 4-byte cp.async copies of its column (copy_tile).  In blocks touching
+// the cube's faces the elements outside, zeros by tensor copies and not copied by row copies, are
+// replaced by the edge values (clamp-to-edge; row copies clamp the rows on the way).  Then:
 //   x-pass: 4(32+2r) threads each make 8 consecutive outputs of a row from at most
 //           six float4 reads, as four packed FP32x2 accumulators (__ffma2_rn rounds
 //           each lane exactly as a scalar FMA, in the same tap order);
@@ -210,15 +211,17 @@ constexpr int smooth_stage_floats()
 }
 
 // One plane of the staged box by 4-byte asynchronous copies (ROWS: a cube whose rows no tensor
-// copy takes), clamped to the edge on the way; 64 threads per row, the thread's own arrival on
-// `bar` once its copies have landed.  src: the plane.
+// copy takes), rows clamped to the edge on the way; 64 threads per row, the thread's own arrival on
+// `bar` once its copies have landed.  src: the plane.  Columns outside the cube are left to the
+// edge clamp: clamped here, up to 45 lanes of a row copied the same element, and such copies go one
+// by one (301 x 300 x 300, r = 8: 320 us, 231 without them; 103 x 298 x 295, r = 1: 75 and 51).
 template <int R>
 __device__ __forceinline__ void copy_tile(float *tile, const float *src, int x0, int y0, int nx, int ny, int tid,
                                           uint64_t *bar)
 {
-    const int c = tid & 63;
-    if (c < kSmBW) {
-        const float *col = src + clampi_s(x0 - kSmXP + c, 0, nx - 1);
+    const int c = tid & 63, x = x0 - kSmXP + c;
+    if (c < kSmBW && x >= 0 && x < nx) {
+        const float *col = src + x;
 #pragma unroll
         for (int row = tid >> 6; row < kSmTY + 2 * R; row += kSmThreads / 64)
             cp_async4(tile + row * kSmBW + c, col + (size_t)clampi_s(y0 - R + row, 0, ny - 1) * nx);
@@ -227,8 +230,8 @@ __device__ __forceinline__ void copy_tile(float *tile, const float *src, int x0,
 }
 
 // ROWS: planes by copy_tile instead of a tensor copy, outputs by elements (a ragged row's
-// column pairs are not aligned).  401 x 300 x 300, r = 6: 247 us, 452 by the kernel without the
-// pipeline (400 x 300 x 300 by tensor copies: 200).
+// column pairs are not aligned).  301 x 300 x 300, r = 6: 208 us, 424 by the kernel without the
+// pipeline.
 template <int R, bool ZIP, bool ROWS>
 __global__ void __launch_bounds__(kSmThreads, smooth_min_blocks<R, ZIP>())
     smooth_tma_kernel(const __grid_constant__ CUtensorMap tmap, const float *__restrict__ in, float *__restrict__ out,
@@ -274,8 +277,9 @@ __global__ void __launch_bounds__(kSmThreads, smooth_min_blocks<R, ZIP>())
     }
     // clamp-to-edge bounds inside the tile (columns / rows that hold real data)
     const int c_lo = max(0, kSmXP - x0), c_hi = min(kSmBW - 1, nx - 1 - (x0 - kSmXP));
-    const int r_lo = max(0, R - y0), r_hi = min(IH - 1, ny - 1 - (y0 - R));
-    const bool edge = !ROWS && (c_lo > 0 || c_hi < kSmBW - 1 || r_lo > 0 || r_hi < IH - 1);
+    // (row copies clamp the rows on the way)
+    const int r_lo = ROWS ? 0 : max(0, R - y0), r_hi = ROWS ? IH - 1 : min(IH - 1, ny - 1 - (y0 - R));
+    const bool edge = c_lo > 0 || c_hi < kSmBW - 1 || r_lo > 0 || r_hi < IH - 1;
 
     // x-pass unit of this thread: row xr, outputs 8 xq .. 8 xq + 7
     const bool xunit = tid < 4 * IH;
@@ -507,9 +511,8 @@ static shw_status smooth_dispatch(const float *in, float *out, int nx, int ny, i
                                   int r, const float *first, cudaStream_t st)
 {
     // the pipeline by tensor copies where their alignment rules hold, by row copies elsewhere; the
-    // staged kernel for radius 0, radii above 8, and ragged cubes of few (x, y) blocks at larger
-    // radii, whose short runs of planes pay for the pipeline's unrolled code (67 x 67 x 510, 9
-    // blocks, r = 6: 60 us staged, 80 by row copies; 127^3, 16 blocks: 70 and 44)
+    // plain kernel for radius 0, radii above 8, and ragged cubes of few (x, y) blocks at larger radii
+    // (67 x 67 x 510, 9 blocks, r = 6: 60 us, 66 by row copies; 127^3, 16 blocks: 70 and 43)
     const bool zip_ok = !ZIP || (aligned(first, 8) && aligned(out, 16));
     // (float2 stores of the tensor-copy form: an 8-byte aligned output)
     const bool tma = nx % 4 == 0 && aligned(in, 16) && zip_ok && aligned(out, 8);
