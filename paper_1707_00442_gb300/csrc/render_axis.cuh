@@ -217,6 +217,12 @@ __device__ __forceinline__ void axis_rows(float *sm, uint64_t *full, uint64_t *e
                 const int wg = A.nx - 4 * np, ws = A.pitch - 4 * np;
 #pragma unroll 4
                 for (int i = lane; i < total; i += 32) {
+                    if constexpr (kChecked) {  // the piece lies in the stage, and in the cube's memory
+                        const long long g = (long long)(b - (unsigned)rz) - A.goff + (ga & ~3);
+                        const bool ok = sa >= 0 && 8 + (sa & ~3) <= A.stage_stride && g >= 0 && g + 4 <= (long long)nvox;
+                        SHW_CHECK(ok);
+                        if (!ok) continue;
+                    }
                     cp_async16(stage + 4 + (sa & ~3), src + (ga & ~3));
                     piece += dpiece;
                     ga += dg;
@@ -231,7 +237,7 @@ __device__ __forceinline__ void axis_rows(float *sm, uint64_t *full, uint64_t *e
                 int row = row0;
                 for (int i = lane; i < total; i += 32) {
                     copy_piece(vol, (unsigned)A.goff, nvox, g0 + (unsigned)(row * A.nx), len, stage,
-                               4 + rz + row * A.pitch, piece);
+                               4 + rz + row * A.pitch, piece, A.stage_stride);
                     piece += dpiece;
                     row += drow;
                     if (piece >= np) {

@@ -214,13 +214,18 @@ __device__ __forceinline__ int floor_div(int a, int b)
 
 // One row's elements [x, x + len) of the cube (len clipped to the row) from row start index
 // `row` into the stage at element index `at` of x: 16-byte pieces by a bulk copy, and at the
-// two ends of the whole cube, where a piece would leave it, single elements.
+// two ends of the whole cube, where a piece would leave it, single elements.  lo, hi: the slot.
 __device__ __forceinline__ void roll_row(const RollArgs &ra, float *stage, long long nvox, long long row, int x, int len,
-                                         int at, uint64_t *bar)
+                                         int at, int lo, int hi, uint64_t *bar)
 {
     const long long g0 = ra.goff + row + x, g1 = g0 + len;  // floats from the 16-byte boundary
     const float *base = ra.cube - ra.goff;
     long long c0 = g0 & ~3LL, c1 = (g1 + 3) & ~3LL;
+    if constexpr (kChecked) {  // whole pieces inside the slot, on 16-byte boundaries there too
+        const bool ok = at + (int)(c0 - g0) >= lo && at + (int)(c1 - g0) <= hi && (at + (int)(c0 - g0)) % 4 == 0;
+        SHW_CHECK(ok);
+        if (!ok) return;
+    }
     bool wrote = false;
     if (c0 < ra.goff) {
         c0 += 4;
@@ -273,6 +278,10 @@ __device__ __forceinline__ void roll_xplanes(const RollArgs &ra, const RollGeom 
 #pragma unroll
         for (int u = 0; u < U; ++u)
             if (at[u] >= 0) {
+                if constexpr (kChecked) {  // inside the plane (the slot holds kRollXG of them)
+                    SHW_CHECK(at[u] < G.plane);
+                    if (at[u] >= G.plane) continue;
+                }
                 slot[at[u]] = v[u].x;
                 slot[at[u] + G.plane] = v[u].y;
                 slot[at[u] + 2 * G.plane] = v[u].z;
@@ -378,7 +387,8 @@ __device__ __forceinline__ bool roll_produce(const TileRays &r, bool persp, cons
                 const int b = sh.ob[ci] + i % G.wb, x = sh.oa[ci];
                 if (b >= n_b) continue;
                 const long long row = M == 2 ? ((long long)c * n[1] + b) * n[0] : ((long long)b * n[1] + c) * n[0];
-                roll_row(ra, stage, nvox, row, x, min(G.wa, n_a - x), sh.pb[ci] + b * G.sb + x, bar);
+                const int lo = (c % G.ns) * G.slot;
+                roll_row(ra, stage, nvox, row, x, min(G.wa, n_a - x), sh.pb[ci] + b * G.sb + x, lo, lo + G.slot, bar);
             }
         }
         if (lane < s) {

@@ -83,12 +83,18 @@ __device__ __forceinline__ void cp_async_arrive(uint64_t *bar)
 // stage[at ...], in the 16-byte pieces that hold them (also the neighbours up to the next
 // 16-byte boundaries); at the two ends of the whole cube, where a piece would leave it, single
 // elements.  goff: floats from the 16-byte boundary below the cube to the cube; (goff + g) and
-// the stage index agree modulo 4 (stage 16-byte aligned).
+// the stage index agree modulo 4 (stage 16-byte aligned, `limit` floats).
 __device__ __forceinline__ void copy_piece(const float *cube, unsigned goff, unsigned nvox, unsigned g, int len,
-                                           float *stage, int at, int j)
+                                           float *stage, int at, int j, int limit)
 {
     const unsigned g0 = goff + g, r = g0 & 3u, c = g0 - r + 4u * (unsigned)j;  // floats from the boundary
     if (4 * j >= (int)r + len) return;
+    if constexpr (kChecked) {  // the piece lies in the stage, at a 16-byte boundary
+        const int d = at - (int)r + 4 * j;
+        const bool ok = d >= 0 && d + 4 <= limit && d % 4 == 0;
+        SHW_CHECK(ok);
+        if (!ok) return;
+    }
     const float *src = cube - goff + c;
     float *dst = stage + at - (int)r + 4 * j;
     if (c >= goff && c + 4u <= goff + nvox) {
