@@ -98,7 +98,9 @@ constexpr size_t kBwdSmem = sizeof(float4) * kLut + sizeof(float) * kBwdWarps * 
 // has its own sums and its lanes add to them in turns: __match_any_sync groups the lanes by
 // entry, each lane's rank in its group is its turn, and the turns (the largest group: 3 to 4)
 // are plain 16-byte loads, adds and stores.  Lanes of a warp therefore step together.  With that
-// 2.68 ms; the voxels of a cell added once per visit and the tiles handed out there and back 1.35 ms.
+// 2.68 ms; the voxels of a cell added once per visit and the tiles handed out there and back 1.37 ms:
+// the warps then wait on the recomputed fetches and the turns, and at the end on the longest rays (6 of
+// 16 cycles an instruction at the last barrier).
 // One CTA of 24 warps per SM, not three of 8: the global sums then take 152 additions each, and
 // their rounding stays below that of one addition per 16 x 16 pixels.
 template <int INTERP, class Idx>

@@ -23,12 +23,15 @@
 // all staged (a footprint wider than the ring's planes) reads global memory; staging decides
 // the speed, never the result.
 //
-// What bounds it (512^3 cube, 1000 x 1000 MIP): with 9 taps per axis the shared-memory pipe (92 %
-// of its wavefronts; 104 corner loads a sample at 2.1 wavefronts each, the conflicts of 32
+// What bounds it (512^3 cube, 1000 x 1000 MIP): with 9 taps per axis the shared-memory pipe (89 %
+// of its cycles; 104 corner loads a sample at 2.2 wavefronts each, the conflicts of 32
 // rays whose cells fall irregularly on 32 banks; 53.9 ms gathered from global memory, 11.5 ms
 // here); with the box issue slots and latency (50 % of issue; 5.86 -> 2.32 ms).  On the way: one
 // lateral range per step instead of one per cell (4 % of the samples in global memory) 16.8 ms;
 // x-major planes as [z][y][4 x] boxes, unspread over the banks (3.9 wavefronts a load) 18.6 ms.
+// All three major axes are in one kernel of 96 registers, which spills (188 to 356 bytes stored for
+// the taps, 140 to 148 for the box), but not where the samples are: 1 of 1200 instructions of that
+// render is a local load or store.
 #pragma once
 
 #include "render_slab.cuh"

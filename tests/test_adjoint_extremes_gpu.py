@@ -76,3 +76,21 @@ def test_checkpoints_without_samples(m):
     for a, b in zip(zero[:2], negative[:2]):
         assert float(a.abs().max()) > 0 and torch.allclose(a, b, rtol=1e-4, atol=1e-6 * float(a.abs().max()))
     assert zero[2] != 0.0 and negative[2] == pytest.approx(zero[2], rel=1e-4)
+
+
+@pytest.mark.parametrize("interp", ["trilinear", "nearest"])
+def test_more_tiles_than_warps(m, interp):
+    """400 x 400 pixels are 5000 tiles, more than the device's 3648 warps: the first come back for a second
+    one, whose gradients and colour-map sums add to the first's.  Tolerance: as for the small cases of
+    test_adjoint_gpu.py."""
+    import oracle
+    dims, s = (32, 32, 32), 0.02
+    cube = scene.diff_cube(dims=dims, n_sources=3)
+    cam = scene.orbit_camera(dims, 30, 20, 400, 400)
+    lut = scene.linear_lut()
+    g = np.random.default_rng(5).normal(size=(400, 400, 4)).astype(np.float32)
+    gv, gl, gs = _backward(m, to_dev(cube), cam, to_dev(lut), to_dev(g), s, interp=interp)
+    _, rv, rl, rs = oracle.render_grad(cube, cam, g.astype(np.float64), interp=interp, lut=lut, opacity_scale=s)
+    assert np.abs(gv.cpu().numpy() - rv).max() <= 1e-4 * np.abs(rv).max()
+    assert np.abs(gl.cpu().numpy() - rl).max() <= 1e-4 * np.abs(rl).max()
+    assert abs(gs - rs) <= 1e-4 * abs(rs)
