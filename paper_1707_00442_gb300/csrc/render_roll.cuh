@@ -29,8 +29,8 @@
 // here); with the box issue slots and latency (50 % of issue; 5.86 -> 2.32 ms).  On the way: one
 // lateral range per step instead of one per cell (4 % of the samples in global memory) 16.8 ms;
 // x-major planes as [z][y][4 x] boxes, unspread over the banks (3.9 wavefronts a load) 18.6 ms.
-// All three major axes are in one kernel of 96 registers, which spills (188 to 356 bytes stored for
-// the taps, 140 to 148 for the box), but not where the samples are: 1 of 1200 instructions of that
+// All three major axes are in one kernel of 96 registers, which spills (208 to 384 bytes stored for
+// the taps, 136 to 144 for the box), but not where the samples are: 1 of 1200 instructions of that
 // render is a local load or store.
 #pragma once
 
@@ -88,6 +88,12 @@ struct RollMaps {
     CUtensorMap m[2];
 };
 
+// Compositing ends a tile when all its rays have stopped.  dead[t % 4]: how many consumer warps need no
+// further step of the CTA's t-th tile, each told once; a hint, so plain shared-memory accesses do.
+// (Told at every stage by the tile's number, as the staged marcher does, the taps' compositing took 3
+// to 15 % longer, and with any report the other modes, whose rays end with the cube, 1 to 4 %.)
+constexpr int kDeadSlots = 4;  // a slot is zeroed when the tiles before the last have been consumed
+
 struct RollShared {
     RollHdr hdr[kRollBars];
     uint64_t full[kRollBars], empty[kRollBars];
@@ -96,7 +102,7 @@ struct RollShared {
     // cell c of a step: the lateral cells [x, x + y) along A and [z, z + w) along B whose
     // corners and taps the planes of its window all hold
     int4 range[kRollTable];
-    int done[kSlabWarps];  // (SlabShared)
+    int dead[kDeadSlots];
     int quit;
     int pad[3];
 };
@@ -192,7 +198,7 @@ struct RollRing {
                 return false;
         return true;
     }
-    __device__ __forceinline__ bool post_plain(int type, int tile)
+    __device__ __forceinline__ bool post_plain(int type, int tile, int seq = 0)
     {
         if (!drain_to(posts - kRollBars)) return false;
         const int st = posts % kRollBars;
@@ -200,6 +206,8 @@ struct RollRing {
             RollHdr h{};
             h.type = type;
             h.tile = tile;
+            h.m0 = seq % kDeadSlots;  // (a tile's start: its entry of sh.dead)
+            if (type == kStageTile) sh.dead[seq % kDeadSlots] = 0;
             sh.hdr[st] = h;
             mbar_arrive(&sh.full[st]);
         }
@@ -293,9 +301,9 @@ __device__ __forceinline__ void roll_xplanes(const RollArgs &ra, const RollGeom 
     }
 }
 
-template <int M>
+template <int M, bool EARLY>
 __device__ __forceinline__ bool roll_produce(const TileRays &r, bool persp, const CUtensorMap *map,
-                                             const RenderArgs &a, const RollArgs &ra, int tile, float *stage,
+                                             const RenderArgs &a, const RollArgs &ra, int tile, int seq, float *stage,
                                              RollRing &ring)
 {
     using AX = RollAxes<M>;
@@ -334,7 +342,10 @@ __device__ __forceinline__ bool roll_produce(const TileRays &r, bool persp, cons
     bool fresh = true;
     int have_lo = 0, have_hi = -1;  // slots staged
     for (int m0 = floor_div(dir > 0 ? first : last, s) * s; dir > 0 ? m0 <= last : m0 + s > first; m0 += dir * s) {
-        if (tile_done(sh.done, tile)) break;  // every ray of the tile has ended
+        if (EARLY) {  // every ray of the tile has ended
+            const int d = *const_cast<const volatile int *>(sh.dead + seq % kDeadSlots);
+            if (__shfl_sync(0xffffffffu, d, 0) == kSlabWarps) break;
+        }
         const int plo = max(m0 - H, 0), phi = min(m0 + s + H, n_m - 1);
         const int slo = plo / g, shi = phi / g;
         const int c0 = fresh ? slo : (dir > 0 ? have_hi + 1 : slo), c1 = fresh ? shi : (dir > 0 ? shi : have_lo - 1);
@@ -429,6 +440,7 @@ __device__ __forceinline__ bool roll_produce(const TileRays &r, bool persp, cons
     return true;
 }
 
+template <bool EARLY>
 __device__ __forceinline__ void roll_producer(const CUtensorMap *maps, const shw_camera &cam, const RenderArgs &a,
                                               const RollArgs &ra, float *stage, RollShared &sh)
 {
@@ -436,7 +448,7 @@ __device__ __forceinline__ void roll_producer(const CUtensorMap *maps, const shw
     RollRing ring{sh, ra};
     const int on[3] = {ra.geo[0].on, ra.geo[1].on, ra.geo[2].on};
     bool ok = true;
-    while (ok) {
+    for (int seq = 0; ok; ++seq) {
         unsigned t = 0;
         if (lane == 0) t = atomicAdd(ra.ctr, 1u);
         t = __shfl_sync(0xffffffffu, t, 0);
@@ -444,17 +456,17 @@ __device__ __forceinline__ void roll_producer(const CUtensorMap *maps, const shw
             ring.post_plain(kStageExit, 0);
             break;
         }
-        if (!ring.post_plain(kStageTile, (int)t)) break;
+        if (!ring.post_plain(kStageTile, (int)t, seq)) break;
         int tx, ty;
         slab_tile((int)t, a, tx, ty);
         const TileRays r = roll_rays(cam, tx * kSlabTW, ty * kSlabTH, on, ra.xbias);
         const bool persp = !cam.ortho;
         if (r.major == 0)
-            ok = roll_produce<0>(r, persp, nullptr, a, ra, (int)t, stage, ring);
+            ok = roll_produce<0, EARLY>(r, persp, nullptr, a, ra, (int)t, seq, stage, ring);
         else if (r.major == 1)
-            ok = roll_produce<1>(r, persp, &maps[0], a, ra, (int)t, stage, ring);
+            ok = roll_produce<1, EARLY>(r, persp, &maps[0], a, ra, (int)t, seq, stage, ring);
         else
-            ok = roll_produce<2>(r, persp, &maps[1], a, ra, (int)t, stage, ring);
+            ok = roll_produce<2, EARLY>(r, persp, &maps[1], a, ra, (int)t, seq, stage, ring);
         if (ok) ok = ring.post_plain(kStageTileEnd, (int)t);
     }
     // no exit while a copy into this CTA's shared memory is in flight: wait (bounded) for the
@@ -678,6 +690,7 @@ __device__ __forceinline__ void roll_consumer(const S &s, const shw_camera &cam,
     long long pix = 0;
     int N = 0;
     bool has = false, live = false;
+    int slot = -1;  // compositing: the tile's entry of sh.dead, -1 once told
     for (int posts = 0;; ++posts) {
         const int si = posts % kRollBars;
         if (!slab_wait(&sh.full[si], (uint32_t)((posts / kRollBars) & 1), quit, ra.err, ra.polls)) return;
@@ -692,6 +705,7 @@ __device__ __forceinline__ void roll_consumer(const S &s, const shw_camera &cam,
             const bool hit = has && !quick_miss(cam, px, py, s.nx, s.ny, s.nz) &&
                              setup_ray(cam, px, py, s.nx, s.ny, s.nz, a.step, r);
             N = hit ? min(r.N, a.nmax) : 0;
+            slot = h.m0;
             live = N > 0;
             q.st = typename RollMarch<MODE, KIND>::St{};
             q.done = 0;
@@ -742,7 +756,11 @@ __device__ __forceinline__ void roll_consumer(const S &s, const shw_camera &cam,
             has = false;
         }
         __syncwarp();
-        report_done(sh.done, sh.hdr[si].tile, live && q.k < q.kend);
+        if constexpr (is_composite<MODE>)
+            if (h.type != kStageTileEnd && slot >= 0 && !__any_sync(0xffffffffu, live && q.k < q.kend)) {
+                if (lane == 0) atomicAdd(sh.dead + slot, 1);
+                slot = -1;
+            }
         if (lane == 0) mbar_arrive(&sh.empty[si]);
     }
 }
@@ -762,13 +780,12 @@ __global__ void __launch_bounds__(kSlabThreads, kRollMinBlocks)
             mbar_init(&sh.full[i], 1);
             mbar_init(&sh.empty[i], kSlabWarps);
         }
-        for (int w = 0; w < kSlabWarps; ++w) sh.done[w] = -1;
         sh.quit = 0;
         fence_barrier_init();
     }
     __syncthreads();
     if ((threadIdx.x >> 5) == kSlabWarps)
-        roll_producer(maps.m, cam, a, ra, stage, sh);
+        roll_producer<is_composite<MODE>>(maps.m, cam, a, ra, stage, sh);
     else
         roll_consumer<MODE, KIND>(s, cam, a, ra, stage, sh, rings);
 }
