@@ -104,8 +104,8 @@ __global__ void __launch_bounds__(32 * (32 / YB)) smooth_kernel(const float *__r
 // each plane goes into a 3-stage shared ring, signalled through mbarriers: one thread issues
 // cp.async.bulk.tensor loads, the box's x start (x0 - 8) keeping the TMA coordinate 16-byte
 // aligned, or every thread 4-byte cp.async copies of its column (copy_tile).  In blocks touching
-// the cube's faces the elements outside, zeros by tensor copies and not copied by row copies, are
-// replaced by the edge values (clamp-to-edge; row copies clamp the rows on the way).  Then:
+// the cube's faces the elements outside arrive as zeros by tensor copies and are replaced by the
+// edge values (clamp-to-edge); row copies clamp on the way, but for a wide right edge.  Then:
 //   x-pass: 4(32+2r) threads each make 8 consecutive outputs of a row from at most
 //           six float4 reads, as four packed FP32x2 accumulators (__ffma2_rn rounds
 //           each lane exactly as a scalar FMA, in the same tap order);
@@ -212,16 +212,17 @@ constexpr int smooth_stage_floats()
 
 // One plane of the staged box by 4-byte asynchronous copies (ROWS: a cube whose rows no tensor
 // copy takes), rows clamped to the edge on the way; 64 threads per row, the thread's own arrival on
-// `bar` once its copies have landed.  src: the plane.  Columns outside the cube are left to the
-// edge clamp: clamped here, up to 45 lanes of a row copied the same element, and such copies go one
-// by one (301 x 300 x 300, r = 8: 320 us, 231 without them; 103 x 298 x 295, r = 1: 75 and 51).
+// `bar` once its copies have landed.  src: the plane.  Only the columns that the x pass reads.  Those
+// outside the cube are clamped too, unless `fill`, which leaves the ones past its right edge to the
+// edge pass: clamped, up to 30 lanes of a row copy the same element, and such copies go one by one
+// (301 x 300 x 300, r = 8: 320 us, 223 without them; 103 x 298 x 295, r = 1: 75 and 51).
 template <int R>
 __device__ __forceinline__ void copy_tile(float *tile, const float *src, int x0, int y0, int nx, int ny, int tid,
-                                          uint64_t *bar)
+                                          bool fill, uint64_t *bar)
 {
     const int c = tid & 63, x = x0 - kSmXP + c;
-    if (c < kSmBW && x >= 0 && x < nx) {
-        const float *col = src + x;
+    if (c >= kSmXP - R && c < kSmXP + kSmTX + R && (x < nx || !fill)) {
+        const float *col = src + clampi_s(x, 0, nx - 1);
 #pragma unroll
         for (int row = tid >> 6; row < kSmTY + 2 * R; row += kSmThreads / 64)
             cp_async4(tile + row * kSmBW + c, col + (size_t)clampi_s(y0 - R + row, 0, ny - 1) * nx);
@@ -263,10 +264,12 @@ __global__ void __launch_bounds__(kSmThreads, smooth_min_blocks<R, ZIP>())
     }
     __syncthreads();
     if (s_bad) return;  // reported in the error word; nothing was issued
+    // row copies: the right edge by the edge pass (a barrier a plane more) where many columns share it
+    const bool fill = ROWS && kSmXP + kSmTX + R - (nx - (x0 - kSmXP)) > 12;
     if (ROWS) {
         for (int s = 0; s < kSmStages && s < nplanes; ++s)
             copy_tile<R>(s_in + s * STAGE_FLOATS, in + (size_t)clampi_s(zfirst + s, 0, nz - 1) * plane, x0, y0, nx, ny,
-                         tid, &bars[s]);
+                         tid, fill, &bars[s]);
     } else if (tid == 0) {
         for (int s = 0; s < kSmStages && s < nplanes; ++s) {
             if (s == skip_plane) continue;  // fault injection: this plane's copy is never issued
@@ -276,8 +279,9 @@ __global__ void __launch_bounds__(kSmThreads, smooth_min_blocks<R, ZIP>())
         }
     }
     // clamp-to-edge bounds inside the tile (columns / rows that hold real data)
-    const int c_lo = max(0, kSmXP - x0), c_hi = min(kSmBW - 1, nx - 1 - (x0 - kSmXP));
-    // (row copies clamp the rows on the way)
+    // (row copies clamp the rest on the way)
+    const int c_lo = ROWS ? 0 : max(0, kSmXP - x0);
+    const int c_hi = ROWS && !fill ? kSmBW - 1 : min(kSmBW - 1, nx - 1 - (x0 - kSmXP));
     const int r_lo = ROWS ? 0 : max(0, R - y0), r_hi = ROWS ? IH - 1 : min(IH - 1, ny - 1 - (y0 - R));
     const bool edge = c_lo > 0 || c_hi < kSmBW - 1 || r_lo > 0 || r_hi < IH - 1;
 
@@ -339,7 +343,7 @@ __global__ void __launch_bounds__(kSmThreads, smooth_min_blocks<R, ZIP>())
         if (ROWS) {
             if (i + kSmStages < nplanes)
                 copy_tile<R>(tile, in + (size_t)clampi_s(zfirst + i + kSmStages, 0, nz - 1) * plane, x0, y0, nx, ny, tid,
-                             &bars[stage]);
+                             fill, &bars[stage]);
         } else if (tid == 0 && i + kSmStages < nplanes) {
             mbar_arrive_expect_tx(&bars[stage], STAGE_BYTES);
             tma_load_3d(tile, &tmap, x0 - kSmXP, y0 - R, min(max(zfirst + i + kSmStages, 0), nz - 1), &bars[stage]);
