@@ -909,18 +909,21 @@ constexpr int render_min_ctas()
     if (two_cubes<MODE>) return INTERP == SHW_NEAREST ? 1 : 10;
     return INTERP == SHW_NEAREST || is_composite<MODE> ? 12 : 1;
 }
-// The form for more CTAs serves views of at least kManyWarps warps' pixels (below, fewer
-// registers only slow each ray: over 254 ratios of two cubes 0.72 to 1.41 of the other form's time
-// below and 0.79 to 1.00 above; 347 nearest and 344 compositing renders 0.70 to 1.41 below, 0.73 to
-// 1.01 above), and cubes that the second-level cache still helps with: above these sizes more rays
-// in flight draw their planes from HBM over and over (the ratio of two 641^3 cubes on 1000 x 1000
-// at yaw 70 4.87 ms, 5.56 with 10 per SM; compositing 1024^3 clipped at yaw 60 6.6 and 14.1).
-constexpr double kManyWarps = 10000.0;
+// The form for more CTAs serves views that many warps' pixels see, fewer where a warp's rays share
+// rows of the cube; below, fewer registers only slow each ray (over 254 ratios of two cubes it took
+// 0.72 to 0.99 of the other form's time where it is taken, 0.74 to 1.39 elsewhere; 425 nearest renders
+// 0.73 to 1.00 and 0.70 to 1.13, 344 compositing ones 0.76 to 1.12 and 0.88 to 1.60).  And it serves
+// cubes that the second-level cache still helps with: above these sizes more rays in flight draw their
+// planes from HBM over and over, unless they share rows (the ratio of two 641^3 cubes on 1000 x 1000 at yaw 70 4.87 ms, 5.56 with 10
+// per SM, at yaw 0 3.15 and 2.49; compositing 1024^3 clipped at yaw 60 6.6 and 14.1).
+// warps: covered_pixels / 32; rows: warp_rows.
 template <int MODE, int INTERP>
-constexpr double render_max_voxels()
+inline bool render_raised(double warps, double rows, double voxels)
 {
-    if (INTERP == SHW_NEAREST) return 1e30;
-    return two_cubes<MODE> ? 67108864.0 : 536870912.0;
+    if (two_cubes<MODE>)
+        return (warps >= 10000.0 && voxels <= 67108864.0) ||
+               (warps >= 2400.0 && voxels >= 1e6 && rows <= (voxels > 67108864.0 ? 4.0 : 2.0));
+    return (warps >= 8000.0 || (warps >= 3500.0 && rows <= 1.0)) && (INTERP == SHW_NEAREST || voxels <= 536870912.0);
 }
 template <int MODE, int INTERP, class S, int SMK = 0, int MINB = render_min_ctas<MODE, INTERP, SMK>()>
 __global__ void __launch_bounds__(kRenderThreads, MINB)
@@ -993,14 +996,43 @@ inline double centre_pitch(const shw_camera &c, int nx, int ny, int nz)
     return 2.0 * c.tan_half_fovy * std::fabs(depth) / len2 / c.height;
 }
 
-// About how many pixels see the cube: its parallel projection at its centre's scale.
+// About how many pixels see the cube: its parallel projection at its centre's scale, no wider and no
+// higher than the image.
 inline double covered_pixels(const shw_camera &c, int nx, int ny, int nz)
 {
-    const double len = std::sqrt((double)c.fwd[0] * c.fwd[0] + (double)c.fwd[1] * c.fwd[1] + (double)c.fwd[2] * c.fwd[2]);
-    const double area = ((double)ny * nz * std::fabs(c.fwd[0]) + (double)nx * nz * std::fabs(c.fwd[1]) +
-                         (double)nx * ny * std::fabs(c.fwd[2])) / len;  // voxels^2
-    const double pitch = centre_pitch(c, nx, ny, nz), all = (double)c.width * c.height;
-    return area < all * pitch * pitch ? area / (pitch * pitch) : all;
+    const double n[3] = {(double)nx, (double)ny, (double)nz};
+    double len2 = 0.0, area = 0.0, across = 0.0, high = 0.0;  // (voxels)
+    for (int k = 0; k < 3; ++k) {
+        len2 += (double)c.fwd[k] * c.fwd[k];
+        area += n[(k + 1) % 3] * n[(k + 2) % 3] * std::fabs(c.fwd[k]);
+        across += n[k] * std::fabs(c.right[k]);
+        high += n[k] * std::fabs(c.up[k]);
+    }
+    area /= std::sqrt(len2);
+    const double pitch = centre_pitch(c, nx, ny, nz);
+    if (!(pitch > 0.0)) return (double)c.width * c.height;  // the eye is level with the centre
+    across = std::min(across, c.width * pitch);
+    high = std::min(high, c.height * pitch);
+    return area < across * high ? area / (pitch * pitch) : across * high / (pitch * pitch);
+}
+
+// Warp tile orientation for a camera (see the layout note at the top).
+inline int warp_shift_for(const shw_camera &c)
+{
+    if (SHW_WARP_SHIFT >= 0) return SHW_WARP_SHIFT;
+    const float rx = c.right[0] < 0 ? -c.right[0] : c.right[0], ux = c.up[0] < 0 ? -c.up[0] : c.up[0];
+    if (rx >= 0.5f && rx >= ux) return 4;
+    if (ux >= 0.5f) return 1;
+    return 3;
+}
+
+// Rows of the cube (along y and z) that a warp's tile spans at its centre: 0 to 1 where its rays
+// share them, in views along z or y, up to 16 and more where the image's long side runs across rows.
+inline double warp_rows(const shw_camera &c, int nx, int ny, int nz)
+{
+    const int ws = warp_shift_for(c);
+    const double r = std::fabs(c.right[1]) + std::fabs(c.right[2]), u = std::fabs(c.up[1]) + std::fabs(c.up[2]);
+    return centre_pitch(c, nx, ny, nz) * (((1 << ws) - 1) * r + ((32 >> ws) - 1) * u);
 }
 
 // Host-side launch for one storage type (instantiated per storage in its own TU).
@@ -1033,7 +1065,7 @@ shw_status launch_render_modes(int mode, int interp, const S &s, const S &s2, co
         if (more_ctas && interp != SHW_NEAREST) g = std::min(g, std::max(tiles / 4, 8LL * nsm));
         kern<<<(unsigned)std::max<long long>(g, 1), block, 0, st>>>(s, s2, cam, a, ctr, nwarp_tiles);
     };
-    const bool many = covered_pixels(cam, s.nx, s.ny, s.nz) >= 32.0 * kManyWarps;
+    const double warps = covered_pixels(cam, s.nx, s.ny, s.nz) / 32.0, rows = warp_rows(cam, s.nx, s.ny, s.nz);
     const double vox = (double)s.nx * s.ny * s.nz;
     if (SMK > 0 && (ctr == nullptr || nsm <= 0)) return SHW_ECUDA;
 #define SHW_LAUNCH(M, I)                                                       \
@@ -1041,8 +1073,8 @@ shw_status launch_render_modes(int mode, int interp, const S &s, const S &s2, co
         if constexpr (SMK > 0)                                                 \
             persistent(render_kernel_persistent<M, I, S, SMK>,                 \
                        resident_per_sm<render_kernel_persistent<M, I, S, SMK>>(), false); \
-        else if (ctr != nullptr && nsm > 0 && render_min_ctas<M, I, 0>() > 1 && many && \
-                 vox <= render_max_voxels<M, I>())                             \
+        else if (ctr != nullptr && nsm > 0 && render_min_ctas<M, I, 0>() > 1 && \
+                 render_raised<M, I>(warps, rows, vox))                        \
             persistent(render_kernel_persistent<M, I, S>,                      \
                        resident_per_sm<render_kernel_persistent<M, I, S>>(), true); \
         else if (ctr != nullptr && nsm > 0)                                    \
@@ -1097,16 +1129,6 @@ shw_status launch_render_modes(int mode, int interp, const S &s, const S &s2, co
 #undef SHW_CASE
 #undef SHW_LAUNCH
     return after_launch();
-}
-
-// Warp tile orientation for a camera (see the layout note at the top).
-inline int warp_shift_for(const shw_camera &c)
-{
-    if (SHW_WARP_SHIFT >= 0) return SHW_WARP_SHIFT;
-    const float rx = c.right[0] < 0 ? -c.right[0] : c.right[0], ux = c.up[0] < 0 ? -c.up[0] : c.up[0];
-    if (rx >= 0.5f && rx >= ux) return 4;
-    if (ux >= 0.5f) return 1;
-    return 3;
 }
 
 // Entry points of the per-storage translation units.

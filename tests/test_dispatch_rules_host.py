@@ -30,11 +30,18 @@ def ask(tmp_path_factory):
 @pytest.mark.parametrize("dims,yaw,W,H,more,plain", [
     ((50, 50, 37), 70, 1000, 1000, 204, 240), ((750, 750, 70), 20, 1000, 1000, 333, 446),
     ((301, 300, 300), 30, 1600, 1600, 2583, 2871),
+    ((641, 641, 641), 0, 500, 500, 1088, 1496), ((641, 641, 641), 70, 1000, 1000, 5560, 4870),
     ((65, 66, 67), 30, 64, 64, 75, 58), ((201, 200, 200), 0, 200, 200, 210, 165),
     ((68, 388, 169), 227, 169, 549, 433, 321), ((419, 52, 107), 172, 132, 753, 113, 81)])
 def test_more_resident_ctas(ask, dims, yaw, W, H, more, plain):
     """Gathered ratios of two cubes, the second compositing: compiled for more resident CTAs, and not."""
     assert ask("many", dims, scene.orbit_camera(dims, yaw, 20, W, H)) == (more < plain)
+
+
+def test_more_resident_ctas_counts_pixels_of_the_image(ask):
+    """Views that show part of a wide cube: 156 and 103 us, 122 and 88."""
+    assert not ask("many", (332, 44, 149), scene.orbit_camera((332, 44, 149), 182.22, -10.72, 396, 892))
+    assert not ask("many", (560, 73, 123), scene.orbit_camera((560, 73, 123), 173.62, 9.86, 182, 1095))
 
 
 @pytest.mark.parametrize("dims,yaw,pitch,W,staged,gathered", [
