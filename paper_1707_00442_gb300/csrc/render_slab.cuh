@@ -761,24 +761,29 @@ shw_status slab_launch_one(const SlabMaps &maps, const S &s, const shw_camera &c
 // Whether staging pays for a float32 cube or pair storage (the gather marcher is the
 // alternative), from the tile at the cube's projected centre where its rays pass its middle.
 // Most samples of a tile whose footprint overflows the staged box read global memory one at a
-// time; but so long as some slabs fit, staging hides more of that than a gather does.  So a view is
-// gathered only where no request measured was slower for it:
+// time; but so long as some slabs fit, staging hides more of that than a gather does, and a gather
+// spreads a small image over more SMs, and stops with the ray in compositing.  So a view is gathered
+// only where no request measured was slower for it:
 //   - the footprint in a slab of one cell overflows a stage (x-major float32 boxes; pairs, whose
 //     x-major rows are half as many cells, from three quarters of one): 200^3 on 256 x 256, yaw 85:
 //     MIP 495 us staged, 189 gathered; just within, 512^3 on 1000 x 1000, 2422 and 3959;
 //   - y- and z-major footprints wider than 66 cells, or for cubes larger than the second-level
-//     cache, which are gathered from HBM, 110 (256^3 on 400 x 400, yaw 60, 44 cells: 238 staged, 425
-//     gathered; 512^3 on 400 x 400, yaw 90, 110 cells: gathering is 1.6 times as fast); pairs wider
-//     than the box of 34, beyond the cache's size only from 2.2 voxels per pixel on;
-//   - below a tenth of a voxel per pixel, where the gathers hit the first-level cache and the stages'
-//     hand-overs cost more (48^3 on 1000 x 1000, compositing: 218 us staged, 179 gathered).
+//     cache, which are gathered from HBM, 110 (100 in compositing) (256^3 on 400 x 400, yaw 60, 44
+//     cells: 238 staged, 425 gathered; 512^3 on 400 x 400, yaw 90, 110 cells: gathering is 1.6 times as
+//     fast); large footprints of few tiles already when they are coarse, in compositing sooner, and
+//     there any that are (512 x 128 x 128 on 128 x 128, yaw 90: MIP 1246 us staged, 301 gathered);
+//     pairs wider than the box of 34, beyond the cache's size only from 2.2 voxels per pixel on;
+//   - below a tenth of a voxel per pixel (a fifth in compositing), where the gathers hit the
+//     first-level cache and the stages' hand-overs cost more (48^3 on 1000 x 1000, compositing: 218 us
+//     staged, 179 gathered).
 // Over 2984 renders (32^3 .. 1024^3 and oblong cubes, 96^2 .. 2000^2, MIP, compositing, the other
-// modes and pairs) this takes 18 % less time than always staging, and its two worst choices took
-// 1.06 and 1.05 times as long.  (The better of the two each time would take 24 % less.)
+// modes and pairs) this takes 21 less time than always staging, the better of the two each time
+// 24 %; its two worst choices took 1.06 and 1.05 times as long as staging.
 template <class G>
-inline bool slab_pays(const shw_camera &c, int nx, int ny, int nz)
+inline bool slab_pays(const shw_camera &c, int nx, int ny, int nz, bool composite)
 {
     const double pitch = centre_pitch(c, nx, ny, nz);
+    const double tiles = covered_pixels(c, nx, ny, nz) / (kSlabTW * kSlabTH);
     if (pitch <= 0.1) return false;
     float px, py;
     project_centre(c, nx, ny, nz, px, py);
@@ -808,7 +813,14 @@ inline bool slab_pays(const shw_camera &c, int nx, int ny, int nz)
             return ceilf(ext[0] / kSlabRows) * kSlabRows * ext[1] * G::kBXx <= (pair ? 0.75f : 1.02f) * G::kStageElems;
         if (2.0f * ext[1] * (float)(ext[0] + 3.0f <= G::kBXn ? G::kBXn : G::kBXw) > (float)G::kStageElems) return false;
         if (pair) return (hbm && pitch < 2.2) || ext[0] <= 34.0f;
-        return ext[0] <= (hbm ? 110.0f : 66.0f);
+        const float area = ext[0] * ext[1];
+        if (hbm && composite)
+            return ext[0] <= 100.0f && pitch <= 3.0 && !(area > 2200.0f && tiles <= 600.0 && pitch > 1.4);
+        if (hbm) return ext[0] <= 110.0f && !(area > 3000.0f && tiles <= 400.0 && pitch > 2.4);
+        if (composite)
+            return pitch > 0.2 && ((ext[0] <= 66.0f && pitch <= 1.7) || tiles > 100.0) &&
+                   !(area > 800.0f && tiles <= 60.0 && pitch > 0.9);
+        return ext[0] <= 66.0f && !(area > 1400.0f && tiles >= 2.0 && tiles <= 108.0 && pitch > 2.0);
     };
     if (r.major == 0) return pays(std::integral_constant<int, 0>{}, ny, nz, nx);
     if (r.major == 1) return pays(std::integral_constant<int, 1>{}, nx, nz, ny);

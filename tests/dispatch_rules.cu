@@ -25,8 +25,9 @@ int main()
         const double warps = covered_pixels(c, n[0], n[1], n[2]) / 32.0, rows = warp_rows(c, n[0], n[1], n[2]);
         const double vox = (double)n[0] * n[1] * n[2];
         if (!std::strcmp(rule, "many")) yes = render_raised<SHW_RATIO, SHW_TRILINEAR>(warps, rows, vox);
-        if (!std::strcmp(rule, "staged")) yes = slab_pays<SlabGeom<ElemF32>>(c, n[0], n[1], n[2]);
-        if (!std::strcmp(rule, "staged_pair")) yes = slab_pays<SlabGeom<ElemF32Pair>>(c, n[0], n[1], n[2]);
+        if (!std::strcmp(rule, "staged")) yes = slab_pays<SlabGeom<ElemF32>>(c, n[0], n[1], n[2], false);
+        if (!std::strcmp(rule, "staged_composite")) yes = slab_pays<SlabGeom<ElemF32>>(c, n[0], n[1], n[2], true);
+        if (!std::strcmp(rule, "staged_pair")) yes = slab_pays<SlabGeom<ElemF32Pair>>(c, n[0], n[1], n[2], false);
         if (!std::strcmp(rule, "rows")) yes = axis_rows_pay(k, SHW_TRILINEAR, c, n[2]);
         if (!std::strcmp(rule, "rows_nearest")) yes = axis_rows_pay(k, SHW_NEAREST, c, n[2]);
         const bool tmaps = n[0] % 4 == 0;

@@ -55,6 +55,16 @@ def test_staged_marcher(ask, dims, yaw, pitch, W, staged, gathered):
     assert ask("staged", dims, scene.orbit_camera(dims, yaw, pitch, W, W)) == (staged < gathered)
 
 
+@pytest.mark.parametrize("rule,dims,yaw,pitch,W,staged,gathered", [
+    ("staged", (64, 64, 512), 60, -30, 128, 151, 62), ("staged", (256, 256, 64), 20, 60, 128, 189, 87),
+    ("staged_composite", (512, 512, 512), 60, -30, 1000, 1381, 2952),
+    ("staged_composite", (128, 512, 256), 45, 45, 1000, 496, 1045),
+    ("staged_composite", (512, 128, 128), 85, 10, 128, 1190, 255)])
+def test_staged_marcher_of_few_tiles(ask, rule, dims, yaw, pitch, W, staged, gathered):
+    """Coarse views of few tiles, which a gather spreads over more SMs, and compositing."""
+    assert ask(rule, dims, scene.orbit_camera(dims, yaw, pitch, W, W)) == (staged < gathered)
+
+
 def test_staged_marcher_of_pairs(ask):
     for dims, yaw, pitch, W, staged, gathered in [((64, 64, 512), 60, -30, 640, 129, 161),
                                                   ((256, 256, 256), 85, 10, 256, 965, 420)]:
