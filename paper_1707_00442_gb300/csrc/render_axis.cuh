@@ -791,22 +791,25 @@ inline bool axis_box(double ext_x, double ext_y, int nx, int mode, AxisArgs &A, 
 
 // Whether the sweep by row copies pays (else the general marcher gathers).  Its producer warps bring
 // one piece per lane, so a plane costs about 1.7 us however small the tile's share of the cube: it
-// wins when the image has enough tiles to fill the device, earliest for the modes whose samples
-// cost least, and never where a gather is one load (nearest sampling) and the sweep's sample is
-// not.  One CTA per SM composites: a second, nearly empty wave (153 to 227 tiles) loses.  Over 757
+// wins when the image has enough tiles to occupy the device, earliest for the modes whose samples
+// cost least and in magnified views, and never where a gather is one load (nearest sampling) and the
+// sweep's sample is not; there a second, nearly empty wave (153 to 227 tiles) loses.  Over 757
 // maps (cubes of 40^2 .. 640^2 and 16 .. 600 planes, images of half to four times that size) the
-// sweep took 0.36 to 1.05 of the general marcher's time where this takes it and 0.46 to 1.66
+// sweep took 0.36 to 1.05 of the general marcher's time where this takes it and 0.66 to 1.68
 // elsewhere (71 x 71 x 300 on 71^2, compositing: 151 us gathered, 213 by row copies; 601 x 601 x 300
 // on 601^2, MIP: 969 and 459).
 inline bool axis_rows_pay(int mode, int interp, const shw_camera &c, int nz)
 {
     const long long tiles = (long long)ceil_div(c.width, kAxTX) * ceil_div(c.height, kAxTY);
     if (nz < 96 && (long long)c.width * c.height < 65536) return false;
+    const long long pixels = (long long)c.width * c.height;
+    const double pitch = 2.0 * c.ortho_half_h / c.height;  // voxels per pixel
     if (interp == SHW_NEAREST)
-        return mode != SHW_COMPOSITE && mode != SHW_MOMENT1 && tiles >= 228 && nz >= 32;
-    if (mode == SHW_MOMENT1) return tiles >= 64 && nz >= 48;
-    if (mode == SHW_COMPOSITE) return nz >= 48 && ((tiles >= 86 && tiles <= 152) || tiles >= 228);
-    return tiles >= 48;
+        return mode != SHW_COMPOSITE && mode != SHW_MOMENT1 && nz >= 24 && pixels >= 110000 &&
+               tiles >= 110 && (tiles <= 152 || tiles >= 228);
+    if (mode == SHW_MOMENT1) return (tiles >= 64 && nz >= 48) || (tiles >= 48 && pitch <= 0.71);
+    if (mode == SHW_COMPOSITE) return pixels >= 60000 && ((tiles >= 86 && nz >= 24) || (tiles >= 20 && pitch <= 0.71));
+    return tiles >= (pitch <= 0.71 ? 20 : 30);
 }
 
 // Launch the sweep for one (mode, interp, direction); FIX selects the fixed box.

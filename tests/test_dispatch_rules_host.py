@@ -84,6 +84,11 @@ def test_sweep_by_row_copies(ask, rule, n, nz, mode, rows, gathered):
     assert ask(rule, (n, n, nz), ortho_axis_camera((n, n, nz), n, n), mode) == (rows < gathered)
 
 
+def test_sweep_by_row_copies_of_magnified_views(ask):
+    for n, nz, W, mode, rows, gathered in [(71, 300, 142, MIP, 166, 209), (131, 97, 262, COMPOSITE, 113, 128)]:
+        assert ask("rows", (n, n, nz), ortho_axis_camera((n, n, nz), W, W), mode) == (rows < gathered)
+
+
 @pytest.mark.parametrize("rule,dims,yaw,pitch,W,ring,gathered", [
     ("taps", (512, 512, 512), 100, 10, 1000, 7873, 82899), ("taps", (512, 512, 512), 30, 20, 1000, 8656, 24064),
     ("taps", (160, 160, 160), 100, 10, 500, 941, 3855), ("taps_composite", (512, 512, 512), 30, 20, 1000, 6667, 16482),
