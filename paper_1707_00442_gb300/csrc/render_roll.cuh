@@ -23,7 +23,7 @@
 // all staged (a footprint wider than the ring's planes) reads global memory; staging decides
 // the speed, never the result.
 //
-// What bounds it (512^3 cube, 1000 x 1000 MIP): with 9 taps per axis the shared-memory pipe (89 %
+// What bounds it (512^3 cube, 1000 x 1000 MIP): with 9 taps per axis the shared-memory pipe (88 %
 // of its cycles; 104 corner loads a sample at 2.2 wavefronts each, the conflicts of 32
 // rays whose cells fall irregularly on 32 banks; 53.9 ms gathered from global memory, 11.5 ms
 // here); with the box issue slots and latency (50 % of issue; 5.86 -> 2.32 ms).  On the way: one
@@ -932,9 +932,10 @@ shw_status roll_launch_one(const RollMaps &maps, const S &s, const shw_camera &c
 // share rows of the cube (y- and z-major views), most in x-major ones and where the cube exceeds the
 // second-level cache (from 3 x 10^7 voxels on).  Compositing's gathers stop with the ray, the ring
 // with the tile.  From the major axis of the tile at the cube's projected centre, the voxels per
-// pixel there and the tiles that see the cube.  Over 2766 renders (32^3 .. 640^3 and oblong cubes,
-// 96^2 .. 1000^2, eleven views and random ones, 3 to 13 taps, boxes of 3 to 9) the ring took 0.10 to
-// 1.04 of the gather's time where this takes it, up to 11 times as long elsewhere (9 taps, 512^3 on
+// pixel there, the rows that a gathering warp spans (warp_rows) and the tiles that see the cube.
+// Over 2472 renders (32^3 .. 640^3 and oblong cubes, 96^2 .. 1000^2, eleven views and random ones, 3
+// to 13 taps, boxes of 3 to 9) the ring took 0.09 to 1.07 of the gather's time in the 472 where this
+// takes it, 0.14 to 11 times as long elsewhere (9 taps, 512^3 on
 // 1000 x 1000: MIP at yaw 30 24.1 ms gathered, 8.7 staged, at yaw 100 82.6 and 7.9, looking down
 // at yaw 20 13.0 and 8.5, compositing 7.1 and 7.4; 129^3 on 128 x 128, MIP along z 0.33 and 0.59).
 template <int KIND>
@@ -942,6 +943,7 @@ inline bool roll_pays(const shw_camera &cam, const int n[3], bool tmaps, int nta
 {
     const double vox = (double)n[0] * n[1] * n[2], pitch = centre_pitch(cam, n[0], n[1], n[2]);
     const double tiles = covered_pixels(cam, n[0], n[1], n[2]) / (kSlabTW * kSlabTH);
+    const double rows = warp_rows(cam, n[0], n[1], n[2]);
     const int least = std::min(n[0], std::min(n[1], n[2]));
     float px, py;
     project_centre(cam, n[0], n[1], n[2], px, py);
@@ -952,18 +954,26 @@ inline bool roll_pays(const shw_camera &cam, const int n[3], bool tmaps, int nta
     const bool big = vox >= 3e7;
     if (KIND == kRollBox) {  // two fetches a sample when gathered: large cubes by tensor copies only
         if (!tmaps || vox < 1e7) return false;
-        if (composite) return big && pitch <= 1.25 && (major == 0 || (major == 2 && tiles >= 450.0));
-        if (big) return pitch <= 1.6;
-        return least >= 100 && (major == 0 ? pitch <= 0.9 : tiles >= 450.0 && pitch <= 0.7);
+        if (major == 0)
+            return composite ? vox >= 2e7 && rows <= 20.0 && pitch <= 2.0 : least >= 80 && rows <= 15.0 && pitch <= 1.6;
+        if (composite)
+            return least >= 80 && pitch <= 1.25 &&
+                   (major == 2 ? tiles >= 450.0 : rows >= 7.0 && rows <= 20.0 && tiles >= 608.0);
+        return pitch <= 2.5 && (major == 2 ? vox >= 2e7 : rows >= 6.0 && least >= 80);
     }
     // few taps and row copies need a larger cube; below 64 voxels on an axis most taps clamp
     if (least < 64 || !((tmaps && ntaps >= 2) || vox >= 2e6)) return false;
     if (composite) {
-        if (!big) return major == 0 && vox >= 3e6 && least >= 100 && pitch <= 0.9;
-        return major == 0 ? pitch <= 1.25 : major == 2 && tiles >= 450.0 && pitch <= 2.5;
+        if (major == 0)
+            return (least >= 80 && vox >= 3e6 && tiles >= 30.0 && rows <= 16.0 && pitch <= 1.6) ||
+                   (least >= 144 && tiles >= 60.0 && pitch <= 2.5);
+        return major == 2 && big && tiles >= 450.0 && pitch <= 2.5;
     }
-    if (big) return pitch <= 2.5 && tiles >= (major == 2 ? 450.0 : 300.0);
-    return major == 0 ? vox >= 2e6 && tiles >= 152.0 && pitch <= 0.9 : tiles >= 608.0 && pitch <= 0.6;
+    if (major == 0)
+        return (least >= 152 && pitch <= 2.5) || (vox >= 2e6 && rows <= 14.0 && pitch <= 1.6) ||
+               (ntaps >= 2 && rows >= 4.5 && rows <= 16.0 && pitch <= 1.2);
+    return (big && pitch <= 2.5 && tiles >= (major == 2 ? 450.0 : 300.0)) ||
+           (rows >= 5.0 && pitch <= 1.1 && tiles >= 30.0) || (tiles >= 450.0 && pitch <= 0.5);
 }
 
 // In-ray smoothing of a float32 cube through the rolling marcher; SHW_EUNSUPPORTED when it

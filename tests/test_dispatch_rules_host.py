@@ -100,3 +100,13 @@ def test_sweep_by_row_copies_of_magnified_views(ask):
 def test_rolling_marcher(ask, rule, dims, yaw, pitch, W, ring, gathered):
     """9 taps, or the box of 3 to 9: the ring, and the gather."""
     assert ask(rule, dims, scene.orbit_camera(dims, yaw, pitch, W, W), 2) == (ring < gathered)
+
+
+@pytest.mark.parametrize("rule,dims,yaw,pitch,W,ring,gathered", [
+    ("taps", (64, 64, 512), 100, 10, 500, 426, 3336), ("taps", (400, 70, 400), 100, 10, 500, 1245, 4965),
+    ("taps_composite", (512, 512, 512), 100, 10, 500, 4151, 16966),
+    ("box", (512, 512, 512), 0, 0, 500, 682, 1178), ("box", (240, 240, 240), 60, -30, 500, 444, 592),
+    ("box_composite", (512, 512, 512), 60, -30, 1000, 2241, 4109)])
+def test_rolling_marcher_where_a_warp_gathers_many_rows(ask, rule, dims, yaw, pitch, W, ring, gathered):
+    cam = scene.orbit_camera(dims, yaw, pitch, W, W, ortho=(yaw == 0))
+    assert ask(rule, dims, cam, 2) == (ring < gathered)
