@@ -820,7 +820,7 @@ inline bool slab_pays(const shw_camera &c, int nx, int ny, int nz, bool composit
         if (composite)
             return pitch > 0.2 && ((ext[0] <= 66.0f && pitch <= 1.7) || tiles > 100.0) &&
                    !(area > 800.0f && tiles <= 60.0 && pitch > 0.9);
-        return ext[0] <= 66.0f && !(area > 1400.0f && tiles >= 2.0 && tiles <= 108.0 && pitch > 2.0);
+        return ext[0] <= 66.0f && !(area > 1400.0f && tiles >= 2.0 && tiles <= 108.0 && pitch > 2.1);
     };
     if (r.major == 0) return pays(std::integral_constant<int, 0>{}, ny, nz, nx);
     if (r.major == 1) return pays(std::integral_constant<int, 1>{}, nx, nz, ny);
