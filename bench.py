@@ -559,7 +559,7 @@ TRAFFIC_PER_LAUNCH: dict = {
     "smooth2": 2387365376 + 2102186240,
     "render_mip": 1850765056 + 19937024,
     "render_avg": 1862723328 + 16973568,
-    "render_composite": 1763378944 + 17127424,
+    "render_composite": 1666251264 + 18685184,
     "render_spectral": 1877628928 + 17221376,
     "render_ratio": 3900478720 + 24024064,
 }
@@ -568,7 +568,7 @@ TRAFFIC_PER_LAUNCH: dict = {
 WARP_INST_PER_SAMPLE: dict = {
     "mip": 2.322,
     "avg": 2.455,
-    "composite": 3.283,
+    "composite": 3.238,
     "spectral": 2.423,
     "ratio": 3.079,
 }

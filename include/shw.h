@@ -328,7 +328,8 @@ shw_status shw_render_backward(const shw_volume *vol, const shw_camera *cam, con
  * call replaces every flag and returns the previous set.  The switches change which
  * kernel serves a request, never what it computes (the fault switches excepted). */
 #define SHW_DEBUG_NO_AXIS_SWEEP 0x1u  /* orthographic spectral-axis views take the general marcher */
-#define SHW_DEBUG_SMOOTH_PLAIN  0x2u  /* smoothing takes its kernel without tensor copies */
+#define SHW_DEBUG_SMOOTH_PLAIN  0x2u  /* smoothing takes its plain kernel, not the pipeline by tensor copies
+                                         or by row copies */
 #define SHW_DEBUG_BOX_DIRECT    0x4u  /* in-ray box smoothing by direct fetches, never the lattice sums */
 #define SHW_DEBUG_NO_STAGING    0x8u  /* general views and in-ray smoothing take the gather marcher, not the
                                          staged or the rolling one */
