@@ -516,7 +516,7 @@ static shw_status smooth_dispatch(const float *in, float *out, int nx, int ny, i
 {
     // the pipeline by tensor copies where their alignment rules hold, by row copies elsewhere; the
     // plain kernel for radius 0, radii above 8, and ragged cubes of few (x, y) blocks at larger radii
-    // (67 x 67 x 510, 9 blocks, r = 6: 60 us, 66 by row copies; 127^3, 16 blocks: 70 and 43)
+    // (67 x 67 x 510, 9 blocks, r = 6: 60 us, 62 by row copies; 127^3, 16 blocks: 70 and 37)
     const bool zip_ok = !ZIP || (aligned(first, 8) && aligned(out, 16));
     // (float2 stores of the tensor-copy form: an 8-byte aligned output)
     const bool tma = nx % 4 == 0 && aligned(in, 16) && zip_ok && aligned(out, 8);
